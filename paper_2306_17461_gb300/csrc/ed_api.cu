@@ -141,10 +141,15 @@ struct TileJob {
     // resident frontier (time slicing, resuming on wider tiles), or null
     int32_t *keep = nullptr;
     int64_t keep_r = 0, t0 = 0, R0 = 0;
+    // wide-band kernel: the frontier of round init_t - 1 as the batch kernel
+    // left it (entry d + init_zero), to start from when t0 is 0; or null
+    const int32_t *init = nullptr;
+    int64_t init_t = 0, init_zero = 0;
     // tile width to start from (diagonals per CTA; 0: what the longest
     // string could need).  Narrow tiles leave most of the SM's unified
     // L1/shared memory to the L1, which holds the rows' string bytes.
     int64_t smax_want = 0;
+    bool wide = false; // on the wide-band kernel (every job of a launch alike)
 };
 
 // What a tile launch left for one pair: its distance (st 0), or ST_WIDE,
@@ -239,6 +244,7 @@ struct ed_ctx {
     int device = 0;
     int num_sms = 0;
     int grid = 0; // CTAs of the tile kernel
+    int wgrid = 0; // CTAs of the wide-band kernel
     int clock_khz = 1;
     int smem_optin = 0; // largest dynamic shared memory of one CTA
     cudaStream_t stream = nullptr;
@@ -247,7 +253,7 @@ struct ed_ctx {
     size_t held = 0;
     // pool
     DevBuf strA, strB, gf, ctl, gctl, slots, halo, pdesc, res, dump, hashA, hashB, scan, qx, qy, qo, bpairs,
-        border, bnext, bfront, keep;
+        border, bnext, bfront, keep, wtiles;
     unsigned long long *h_res = nullptr; // pinned result block
     size_t h_res_cap = 0;
     uint64_t hash_base = 0;
@@ -442,12 +448,22 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
 {
     int r;
     const int np = (int)jobs.size();
+    const bool wide = jobs[0].wide;
+    int maxg = wide ? ctx->wgrid : ctx->grid;
+    if (wide) { // no more CTAs than the memory budget has room for their tiles
+        int64_t nm = 1;
+        for (const TileJob &j : jobs)
+            nm = std::max(nm, std::max(j.n, j.m));
+        const size_t per = sizeof(int32_t) * lv_wide_tile_words((int)std::min<int64_t>(SMAX_LIMIT, 2 * nm + 2));
+        while (maxg > 1 && per * maxg > ctx->wtiles.bytes && ctx->held - ctx->wtiles.bytes + per * maxg > ctx->budget)
+            maxg = (maxg + 1) / 2;
+    }
     const int h = ctx->eff.block_rounds;
     const int s0 = ctx->eff.tile_width;
     // classes, ascending group size; pairs by class, then cost, largest first
     std::vector<int> sizes;
     for (const TileJob &j : jobs)
-        sizes.push_back(std::max(1, std::min(j.G, ctx->grid)));
+        sizes.push_back(std::max(1, std::min(j.G, maxg)));
     std::vector<int> Gs = sizes;
     std::sort(Gs.begin(), Gs.end());
     Gs.erase(std::unique(Gs.begin(), Gs.end()), Gs.end());
@@ -479,7 +495,7 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
     }
     int used = 0;
     for (int c = ncls - 1; c >= 0; c--)
-        if (used + Gs[c] <= ctx->grid) {
+        if (used + Gs[c] <= maxg) {
             ng[c] = 1;
             used += Gs[c];
         }
@@ -487,7 +503,7 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
         int best = -1;
         double bw = -1.0;
         for (int c = 0; c < ncls; c++)
-            if (ng[c] > 0 && ng[c] < npc[c] && used + Gs[c] <= ctx->grid && wc[c] / ng[c] > bw) {
+            if (ng[c] > 0 && ng[c] < npc[c] && used + Gs[c] <= maxg && wc[c] / ng[c] > bw) {
                 bw = wc[c] / ng[c];
                 best = c;
             }
@@ -539,7 +555,8 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
     if ((r = ensure(ctx, ctx->gf, sizeof(int32_t) * (size_t)std::max<int64_t>(gf_total, 1))) != ED_OK ||
         (r = ensure(ctx, ctx->ctl, sizeof(LaunchCtl))) != ED_OK ||
         (r = ensure(ctx, ctx->gctl, sizeof(GroupCtl) * ngroups)) != ED_OK ||
-        (r = ensure(ctx, ctx->slots, sizeof(JobSlot) * grid * JOB_RING)) != ED_OK ||
+        (wide && (r = ensure(ctx, ctx->wtiles, sizeof(int32_t) * grid * lv_wide_tile_words((int)smax))) != ED_OK) ||
+        (!wide && (r = ensure(ctx, ctx->slots, sizeof(JobSlot) * grid * JOB_RING)) != ED_OK) ||
         (r = ensure(ctx, ctx->halo, sizeof(unsigned long long) * (size_t)grid * 4 * HMAX)) != ED_OK ||
         (r = ensure(ctx, ctx->pdesc, sizeof(PairDesc) * np)) != ED_OK ||
         (r = ensure(ctx, ctx->res, sizeof(unsigned long long) * R_COUNT * np)) != ED_OK)
@@ -571,6 +588,9 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
         pd[q].keep_r = j.keep_r;
         pd[q].t0 = j.t0;
         pd[q].R0 = j.R0;
+        pd[q].init = j.init;
+        pd[q].init_t = j.init_t;
+        pd[q].init_zero = j.init_zero;
     }
     P.pairs = (const PairDesc *)ctx->pdesc.p;
     P.npairs = np;
@@ -579,6 +599,7 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
     P.slots = (JobSlot *)ctx->slots.p;
     P.halo = (unsigned long long *)ctx->halo.p;
     P.gf = (int32_t *)ctx->gf.p;
+    P.wide = (int32_t *)ctx->wtiles.p;
     P.kcap = (int32_t)kcap;
     P.smax = (int32_t)smax;
     P.h = h;
@@ -596,16 +617,17 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
     // bulk-copy staging of long-slide chunks (two stages: the owner streams
     // its first chunks with the next one's copies in flight) when the tiles
     // leave room for it
-    P.stage = lv_tiles_smem_bytes((int)smax, h, 2) <= (size_t)ctx->smem_optin
+    P.stage = wide ? 0 : lv_tiles_smem_bytes((int)smax, h, 2) <= (size_t)ctx->smem_optin
                   ? 2
                   : (lv_tiles_smem_bytes((int)smax, h, 1) <= (size_t)ctx->smem_optin ? 1 : 0);
     CK(cudaMemcpyAsync(ctx->pdesc.p, pd.data(), sizeof(PairDesc) * np, cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(ctx->ctl.p, 0, sizeof(LaunchCtl), s));
     CK(cudaMemsetAsync(ctx->gctl.p, 0, sizeof(GroupCtl) * ngroups, s));
-    CK(cudaMemsetAsync(ctx->slots.p, 0, sizeof(JobSlot) * grid * JOB_RING, s));
+    if (!wide)
+        CK(cudaMemsetAsync(ctx->slots.p, 0, sizeof(JobSlot) * grid * JOB_RING, s));
     CK(cudaMemsetAsync(ctx->res.p, 0, sizeof(unsigned long long) * R_COUNT * np, s));
     CK(cudaEventRecord(ctx->ev0, s));
-    CK(launch_lv_tiles(P, grid, s));
+    CK(wide ? launch_lv_wide(P, grid, s) : launch_lv_tiles(P, grid, s));
     CK(cudaEventRecord(ctx->ev1, s));
     CK(cudaMemcpyAsync(ctx->h_res, ctx->res.p, sizeof(unsigned long long) * R_COUNT * np,
                        cudaMemcpyDeviceToHost, s));
@@ -632,18 +654,18 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
         const unsigned long long *R = ctx->h_res + (size_t)R_COUNT * q;
         TileOut &o = out[i];
         o.st = (uint32_t)R[R_STATUS];
+        const int64_t from = jobs[i].t0 > 0 ? jobs[i].t0 : jobs[i].init ? jobs[i].init_t : 0; // first round run
+        const uint64_t before = from > 0 ? count_extensions(jobs[i].n, jobs[i].m, from - 1) : 0;
         if (o.st == ST_SUSPENDED || (o.st == ST_WIDE && R[R_RESUME_T] > 0)) {
             o.rt = (int64_t)R[R_RESUME_T];
             o.rr = (int64_t)R[R_RESUME_R];
-            // rounds t0 .. rt - 1 done in this launch
-            ctx->last.extensions += count_extensions(jobs[i].n, jobs[i].m, o.rt - 1) -
-                                    (jobs[i].t0 > 0 ? count_extensions(jobs[i].n, jobs[i].m, jobs[i].t0 - 1) : 0);
+            // rounds from .. rt - 1 done in this launch
+            ctx->last.extensions += count_extensions(jobs[i].n, jobs[i].m, o.rt - 1) - before;
         } else if (o.st != 0) {
             continue;
         } else {
             o.k = R[R_K];
-            ctx->last.extensions += count_extensions(jobs[i].n, jobs[i].m, (int64_t)R[R_K]) -
-                                    (jobs[i].t0 > 0 ? count_extensions(jobs[i].n, jobs[i].m, jobs[i].t0 - 1) : 0);
+            ctx->last.extensions += count_extensions(jobs[i].n, jobs[i].m, (int64_t)R[R_K]) - before;
         }
         ctx->last.slide_chars += R[R_SLIDE];
         ctx->last.compared_bytes += 2ull * (R[R_SLIDE] + R[R_MISMATCH]);
@@ -681,17 +703,18 @@ int run_tiles(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStream_t s, std
         std::vector<TileJob> next;
         std::vector<size_t> nidx;
         for (size_t i = 0; i < cur.size(); i++) {
+            const int maxg = cur[i].wide ? ctx->wgrid : ctx->grid;
             if (o[i].st == 0) {
                 k[idx[i]] = o[i].k;
             } else if (o[i].st == ST_WIDE &&
-                       (cur[i].G < ctx->grid || (cur[i].smax_want > 0 && cur[i].smax_want < SMAX_LIMIT))) {
+                       (cur[i].G < maxg || (cur[i].smax_want > 0 && cur[i].smax_want < SMAX_LIMIT))) {
                 // wider tiles first, then a larger group; from the saved
                 // round when the kernel left one in the pair's keep buffer
                 TileJob j = cur[i];
                 if (j.smax_want > 0 && j.smax_want < SMAX_LIMIT)
                     j.smax_want = std::min<int64_t>(SMAX_LIMIT, 4 * j.smax_want);
                 else
-                    j.G = std::min(ctx->grid, 2 * std::max(1, j.G));
+                    j.G = std::min(maxg, 2 * std::max(1, j.G));
                 const bool resume = j.keep && o[i].rt > 0;
                 j.t0 = resume ? o[i].rt : 0;
                 j.R0 = resume ? o[i].rr : 0;
@@ -843,6 +866,7 @@ int ed_create(ed_ctx **out, const ed_config *cfg)
     // co-resident grid for the cooperative tile kernel: one 512-thread CTA per SM
     c->grid = c->cfg.grid_ctas > 0 ? std::min(c->cfg.grid_ctas, c->num_sms) : c->num_sms;
     c->grid = std::min(c->grid, MAX_GRID);
+    c->wgrid = std::min(c->cfg.grid_ctas > 0 ? c->grid : WIDE_PER_SM * c->num_sms, MAX_GRID);
     CK(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
     CK(cudaEventCreate(&c->ev0));
     CK(cudaEventCreate(&c->ev1));
@@ -870,7 +894,7 @@ int ed_destroy(ed_ctx *ctx)
                       &ctx->halo,  &ctx->pdesc,  &ctx->res,   &ctx->dump,   &ctx->hashA,     &ctx->hashB,
                       &ctx->scan,  &ctx->qx,     &ctx->qy,    &ctx->qo,     &ctx->bpairs,    &ctx->border,
                       &ctx->bnext, &ctx->bfront, &ctx->arena_buf, &ctx->s_pairs, &ctx->s_order, &ctx->s_next,
-                      &ctx->keep};
+                      &ctx->keep,  &ctx->wtiles};
     for (DevBuf *b : bufs)
         release(ctx, *b);
     if (ctx->h_res)
@@ -1216,11 +1240,12 @@ static int batch_launch(ed_ctx *ctx, std::vector<BatchPair> &hp, const std::vect
 }
 
 // A tile job for a pair parked by the batch kernel after t rounds with its
-// furthest row at `reach`.  Its distance is estimated by extrapolating the
-// rounds per row so far (t * n / reach, between t and max(n, m)); its group
-// is the smallest power of two of CTAs whose tiles hold that band with a
-// quarter to spare.  The estimate only places the pair: one whose band
-// outgrows its group runs again on a larger group.
+// furthest row at `reach`: it goes on from there on the wide-band kernel.  Its
+// distance is estimated by extrapolating the rounds per row so far (t * n /
+// reach, between t and max(n, m)); its group is the smallest power of two of
+// CTAs whose tiles hold that band with a quarter to spare.  The estimate only
+// places the pair: one whose band outgrows its group runs again on a larger
+// group.
 static TileJob parked_job(ed_ctx *ctx, const BatchPair &b)
 {
     const int64_t nm = std::max(b.n, b.m);
@@ -1228,38 +1253,71 @@ static TileJob parked_job(ed_ctx *ctx, const BatchPair &b)
     int64_t kest = b.reach > 0 ? (int64_t)((double)t * (double)b.n / (double)b.reach) : nm;
     kest = std::min(std::max(kest, t), nm);
     TileJob j{b.A, b.B, b.n, b.m, nullptr, nullptr, nullptr, 0, 1, (double)kest};
+    j.wide = true;
+    j.init = b.front;
+    j.init_t = b.t + 1;
+    j.init_zero = BATCH_W / 2 + 1;
     const int64_t band = std::min<int64_t>(2 * (kest + kest / 4) + 1, b.n + b.m + 1);
-    while (j.G < ctx->grid && (int64_t)j.G * SMAX_LIMIT < band)
+    while (j.G < ctx->wgrid && (int64_t)j.G * SMAX_LIMIT < band)
         j.G *= 2;
-    j.G = std::min(j.G, ctx->grid);
+    j.G = std::min(j.G, ctx->wgrid);
     return j;
 }
 
-// While the groups the jobs ask for fill at most half of the grid, doubles
-// them: with few pairs, more CTAs per pair shorten each round; a single job
-// takes the whole grid.  The cost of a job (for sharing CTAs among classes)
-// is its estimated distance times the round time, which grows with the band
-// per CTA.
+// Sizes the groups of wide-band jobs (G at least what each band needs; cost:
+// the estimated distance k on entry, the estimated run time in microseconds
+// on return).  A round on a group of G CTAs takes about WIDE_ROUND_US (the
+// chain along the alignment path) and WIDE_DIAG_US for each diagonal of the
+// band's share, about k / G on average.  Small groups waste least of the
+// chain, but the longest job bounds the launch: a job that would take more
+// than half of what the whole set takes on all CTAs (one and a half times
+// that while the groups leave CTAs free) gets a group twice as large, down to
+// WIDE_TILE_MIN diagonals a CTA.  A single job takes the whole grid, and while
+// the groups fill at most half of it they are doubled.
+constexpr double WIDE_ROUND_US = 2.0, WIDE_DIAG_US = 0.75e-3;
+constexpr int64_t WIDE_TILE_MIN = 512;
 static void spread_jobs(ed_ctx *ctx, std::vector<TileJob> &jobs)
 {
     if (jobs.size() == 1)
-        jobs[0].G = ctx->grid;
+        jobs[0].G = ctx->wgrid;
+    auto time = [](const TileJob &j) {
+        const double width = std::min(j.cost, 0.5 * (double)(j.n + j.m + 1)); // mean band width
+        return j.cost * (WIDE_ROUND_US + WIDE_DIAG_US * width / (double)j.G);
+    };
+    auto wider = [&](const TileJob &j) {
+        const int64_t band = std::min<int64_t>((int64_t)(2.0 * j.cost) + 1, j.n + j.m + 1);
+        return j.G < ctx->wgrid && band / (2 * j.G) >= WIDE_TILE_MIN;
+    };
+    for (bool more = jobs.size() > 1; more;) {
+        more = false;
+        double total = 0.0;
+        int64_t sum = 0;
+        for (const TileJob &j : jobs) {
+            total += time(j) * j.G;
+            sum += j.G;
+        }
+        const double share = (sum > ctx->wgrid ? 0.5 : 1.5) * total / ctx->wgrid;
+        for (TileJob &j : jobs)
+            if (time(j) > share && wider(j)) {
+                j.G = std::min(ctx->wgrid, 2 * j.G);
+                more = true;
+            }
+    }
     for (;;) {
         int64_t sum = 0;
         bool room = false;
         for (const TileJob &j : jobs) {
             sum += j.G;
-            room |= j.G < ctx->grid;
+            room |= wider(j);
         }
-        if (!room || 2 * sum > ctx->grid)
+        if (!room || 2 * sum > ctx->wgrid)
             break;
         for (TileJob &j : jobs)
-            j.G = std::min(ctx->grid, 2 * j.G);
+            if (wider(j))
+                j.G = std::min(ctx->wgrid, 2 * j.G);
     }
-    for (TileJob &j : jobs) {
-        const double band = std::min(2.0 * j.cost + 1.0, (double)(j.n + j.m + 1));
-        j.cost = j.cost * (1.0 + band / ((double)j.G * 4096.0));
-    }
+    for (TileJob &j : jobs)
+        j.cost = time(j);
 }
 
 static int batch_core(ed_ctx *ctx, size_t np, const uint8_t *const *A, const size_t *n,
@@ -1307,8 +1365,13 @@ static int batch_core(ed_ctx *ctx, size_t np, const uint8_t *const *A, const siz
         // pairs whose band outgrew one CTA: CTA groups of the tile kernel,
         // sized by each pair's estimated distance, in one launch
         std::vector<TileJob> jobs;
-        for (size_t p : parked)
-            jobs.push_back(parked_job(ctx, hp[p]));
+        for (size_t p : parked) {
+            const BatchPair &b = hp[p];
+            jobs.push_back(parked_job(ctx, b));
+            ext += count_extensions(b.n, b.m, b.t); // its rounds so far
+            slide += b.slide;
+            mism += b.mism;
+        }
         spread_jobs(ctx, jobs);
         ctx->last = ed_stats{};
         std::vector<uint64_t> kk;
@@ -1413,7 +1476,7 @@ static void to_tiles(ed_ctx *ctx, Request *q, int G)
 {
     ctx->arena.release(q->keep, q->bytesK);
     q->tile_G = G;
-    q->keep_r = std::min<int64_t>(std::max(q->n, q->m), (int64_t)ctx->grid * SMAX_LIMIT);
+    q->keep_r = std::min<int64_t>(std::max(q->n, q->m), (int64_t)ctx->wgrid * SMAX_LIMIT);
     q->bytesK = sizeof(int32_t) * (size_t)(2 * q->keep_r + 5);
     q->keep = ctx->arena.alloc(q->bytesK);
     q->t0 = 0;
@@ -1492,6 +1555,7 @@ static void engine_loop(ed_ctx *ctx)
                     // the group its estimated band needs; each step spreads
                     // the groups over the grid
                     const TileJob pj = parked_job(ctx, b);
+                    q->t = b.t;
                     q->cost = pj.cost;
                     to_tiles(ctx, q, pj.G);
                 } else {
@@ -1509,10 +1573,14 @@ static void engine_loop(ed_ctx *ctx)
                 continue;
             TileJob j{(const uint8_t *)q->dA, (const uint8_t *)q->dB, q->n, q->m, nullptr, nullptr, nullptr, 0,
                       q->tile_G, q->cost};
+            j.init = (const int32_t *)q->front;
+            j.init_t = q->t + 1;
+            j.init_zero = BATCH_W / 2 + 1;
             j.keep = (int32_t *)q->keep;
             j.keep_r = q->keep ? q->keep_r : 0;
             j.t0 = q->keep ? q->t0 : 0;
             j.R0 = q->R0;
+            j.wide = true;
             tidx.push_back(i);
             jobs.push_back(j);
         }
@@ -1536,13 +1604,13 @@ static void engine_loop(ed_ctx *ctx)
                     q->t0 = o[j].rt;
                     q->R0 = o[j].rr;
                     ctx->n_slices++;
-                } else if (o[j].st == ST_WIDE && q->keep && o[j].rt > 0 && jobs[j].G < ctx->grid) {
+                } else if (o[j].st == ST_WIDE && q->keep && o[j].rt > 0 && jobs[j].G < ctx->wgrid) {
                     // a larger group from the saved round
-                    q->tile_G = std::min(ctx->grid, 2 * jobs[j].G);
+                    q->tile_G = std::min(ctx->wgrid, 2 * jobs[j].G);
                     q->t0 = o[j].rt;
                     q->R0 = o[j].rr;
-                } else if (o[j].st == ST_WIDE && q->tile_G < ctx->grid) {
-                    to_tiles(ctx, q, std::min(ctx->grid, 2 * q->tile_G)); // again, from round 0
+                } else if (o[j].st == ST_WIDE && q->tile_G < ctx->wgrid) {
+                    to_tiles(ctx, q, std::min(ctx->wgrid, 2 * q->tile_G)); // again, from round 0
                 } else {
                     result[tidx[j]] = ED_ELIMIT;
                     done[tidx[j]] = 1;

@@ -13,6 +13,8 @@ constexpr uint32_t ST_WIDE = 8;   // per pair: the band outgrew its group's tile
 constexpr uint32_t ST_SUSPENDED = 9; // per pair: budget spent, frontier saved to keep
 
 constexpr int CTA_THREADS = 256;   // threads of a tile CTA (up to 255 registers each)
+constexpr int WIDE_THREADS = 512; // threads of a wide-band CTA (128 registers each)
+constexpr int WIDE_PER_SM = 1;    // its CTAs per SM
 constexpr int MAX_GRID = 1024;     // CTAs of one tile launch, at most
 constexpr int HMAX = 64;           // rounds per temporal block, at most
 constexpr int CHUNK_BYTES = 16 * 1024; // bytes of one job-slot claim (per string)
@@ -53,6 +55,10 @@ struct PairDesc {
     // with epoch radius R0 when t0 > 0
     int32_t *keep;
     int64_t keep_r, t0, R0;
+    // wide-band kernel, t0 = 0: the frontier of round init_t - 1 to start
+    // from, L[d] at init[d + init_zero] for |d| < init_t; or null
+    const int32_t *init;
+    int64_t init_t, init_zero;
 };
 
 // Per group of CTAs (zeroed before the launch).
@@ -144,10 +150,15 @@ struct LvArgs {
     // slide's chunks (0: loads into registers instead; 2: the owner streams
     // its first chunks with the next one's copies in flight)
     int32_t stage;
+    int32_t *wide; // the wide-band kernel's tiles: gridDim.x * lv_wide_tile_words(smax)
 };
 
 size_t lv_tiles_smem_bytes(int smax, int h, int stage);
 cudaError_t launch_lv_tiles(const LvArgs &P, int grid, cudaStream_t s);
+// The wide-band kernel (lv_wide.cu): the same arguments (slots, hash, dump and
+// help fields unused); direct comparison only.
+size_t lv_wide_tile_words(int smax); // int32 words of LvArgs::wide per CTA
+cudaError_t launch_lv_wide(const LvArgs &P, int grid, cudaStream_t s);
 
 // ---------------------------------------------------------------- batch
 // One pair of a batch / serving slot.  Frontier state lives in global
