@@ -222,26 +222,24 @@ int ed_lcp_dev(ed_ctx *ctx, const uint8_t *A, size_t n, const uint8_t *B,
 
 /* The prefix table of Sec. 3.2: T[i] = sum_{j<i} (X[j]+1) * p^(i-1-j)
  * mod 2^61-1 for i = 0..len, p = ed_hash_base(ctx).  X and T are device
- * pointers; T has len + 1 uint64 entries.  One single-pass scan launch;
- * synchronous on `stream`.  ED_ETIMEOUT when a bounded wait of the scan
- * gave up (the table is then not valid). */
+ * pointers; T has len + 1 uint64 entries.  One launch up to 16384 bytes, else
+ * three (tile hashes, their scan, the table); synchronous on `stream`. */
 int ed_prefix_hash_dev(ed_ctx *ctx, const uint8_t *X, size_t len, uint64_t *T,
                        void *stream);
 
 /* The blocked prefix table of Sec. 3.3 (Alg. 2): T[j] = h(X[0..j*b)) for
  * j = 0..len/b, the entries of ed_prefix_hash_dev's table at multiples of
  * b (1 <= b <= 2^20).  X and T are device pointers; T has len/b + 1 uint64
- * entries.  One scan launch that writes only the block prefixes.
- * Synchronous on `stream`; ED_ETIMEOUT as for ed_prefix_hash_dev. */
+ * entries.  The launches of ed_prefix_hash_dev, which then write only the
+ * block prefixes.  Synchronous on `stream`. */
 int ed_prefix_hash_blocked_dev(ed_ctx *ctx, const uint8_t *X, size_t len, size_t b, uint64_t *T,
                                void *stream);
 
 /* The hash base p used by the context (derived from hash_seed). */
 uint64_t ed_hash_base(ed_ctx *ctx);
 
-/* Largest len accepted by ed_prefix_hash_noalloc (21843 scan tiles of 4096
- * bytes: the scan's 48-byte look-back descriptors plus a 64-byte header fit
- * its 1 MiB scratch array). */
+/* Largest len accepted by ed_prefix_hash_noalloc (the hashes of its
+ * scan tiles fit the library's 1 MiB scratch array many times over). */
 #define ED_NOALLOC_MAX_LEN ((size_t)89468928)
 
 /* ed_prefix_hash_dev for callers that cannot allocate device memory: code
@@ -262,8 +260,7 @@ uint64_t ed_hash_base(ed_ctx *ctx);
  * call before any stream capture).  Every call shares the array and clears
  * it on `stream` before use: calls whose work overlaps on the GPU (two
  * streams, or two threads) race and must be serialised by the caller.
- * Synchronous on `stream` (NULL = legacy default).  ED_ETIMEOUT when a
- * bounded wait of the scan gave up (the table is then not valid). */
+ * Synchronous on `stream` (NULL = legacy default). */
 int ed_prefix_hash_noalloc(const uint8_t *X, size_t len, uint64_t base, uint64_t *T,
                            void *stream);
 

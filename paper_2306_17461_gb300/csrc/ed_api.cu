@@ -397,22 +397,6 @@ void resolve(ed_ctx *ctx, int64_t n, int64_t m, bool single)
     ctx->eff = e;
 }
 
-// Waits for the prefix-hash scan last launched on s with the context's scan
-// state and maps its status word: a look-back wait that gave up leaves a
-// wrong table, reported as ED_ETIMEOUT.
-int scan_result(ed_ctx *ctx, cudaStream_t s)
-{
-    cudaError_t e = cudaSuccess;
-    const uint32_t st = prefix_hash_status(ctx->scan.p, s, &e);
-    if (e != cudaSuccess)
-        return cuda_fail(ctx, e, "prefix hash scan");
-    if (st != 0) {
-        ctx->last_err = "prefix hash scan: a look-back wait gave up";
-        return status_from_kernel(st);
-    }
-    return ED_OK;
-}
-
 int run_hash_tables(ed_ctx *ctx, const uint8_t *dA, int64_t n, const uint8_t *dB, int64_t m,
                     cudaStream_t s)
 {
@@ -425,14 +409,8 @@ int run_hash_tables(ed_ctx *ctx, const uint8_t *dA, int64_t n, const uint8_t *dB
     const size_t sb = std::max(prefix_hash_state_bytes(n), prefix_hash_state_bytes(m));
     if ((r = ensure(ctx, ctx->scan, sb)) != ED_OK)
         return r;
-    CK(launch_prefix_hash(dA, n, ctx->hash_base, (uint64_t *)ctx->hashA.p, b, ctx->scan.p,
-                          prefix_hash_state_bytes(n), s));
-    if ((r = scan_result(ctx, s)) != ED_OK)
-        return r;
-    CK(launch_prefix_hash(dB, m, ctx->hash_base, (uint64_t *)ctx->hashB.p, b, ctx->scan.p,
-                          prefix_hash_state_bytes(m), s));
-    if ((r = scan_result(ctx, s)) != ED_OK)
-        return r;
+    CK(launch_prefix_hash(dA, n, ctx->hash_base, (uint64_t *)ctx->hashA.p, b, ctx->scan.p, s));
+    CK(launch_prefix_hash(dB, m, ctx->hash_base, (uint64_t *)ctx->hashB.p, b, ctx->scan.p, s));
     ctx->last.kernel_launches += 2;
     return ED_OK;
 }
@@ -1106,8 +1084,9 @@ int ed_prefix_hash_dev(ed_ctx *ctx, const uint8_t *X, size_t len, uint64_t *T, v
     if ((r = ensure(ctx, ctx->scan, sb)) != ED_OK)
         return r;
     cudaStream_t s = (cudaStream_t)stream;
-    CK(launch_prefix_hash(X, (int64_t)len, ctx->hash_base, T, 1, ctx->scan.p, sb, s));
-    return scan_result(ctx, s);
+    CK(launch_prefix_hash(X, (int64_t)len, ctx->hash_base, T, 1, ctx->scan.p, s));
+    CK(cudaStreamSynchronize(s));
+    return ED_OK;
 }
 
 int ed_prefix_hash_blocked_dev(ed_ctx *ctx, const uint8_t *X, size_t len, size_t b, uint64_t *T, void *stream)
@@ -1121,8 +1100,9 @@ int ed_prefix_hash_blocked_dev(ed_ctx *ctx, const uint8_t *X, size_t len, size_t
     if ((r = ensure(ctx, ctx->scan, sb)) != ED_OK)
         return r;
     cudaStream_t s = (cudaStream_t)stream;
-    CK(launch_prefix_hash(X, (int64_t)len, ctx->hash_base, T, (int64_t)b, ctx->scan.p, sb, s));
-    return scan_result(ctx, s);
+    CK(launch_prefix_hash(X, (int64_t)len, ctx->hash_base, T, (int64_t)b, ctx->scan.p, s));
+    CK(cudaStreamSynchronize(s));
+    return ED_OK;
 }
 
 int ed_lcp_dev(ed_ctx *ctx, const uint8_t *A, size_t n, const uint8_t *B, size_t m, const int64_t *x,

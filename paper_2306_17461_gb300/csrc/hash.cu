@@ -1,205 +1,342 @@
-// hash.cu -- the prefix-hash table of Sec. 3.2 built by one single-pass
-// scan on the device.
+// hash.cu -- the prefix-hash table of Sec. 3.2 on the device.
 //
 //   T[i] = h(X[0..i)) = sum_{j<i} (X[j] + 1) * p^(i-1-j)   mod q = 2^61 - 1
 //
 // Prefix hashes compose by the concatenation rule of Sec. 2,
-//   (h1, P1) (+) (h2, P2) = (h1 * P2 + h2, P1 * P2),  P = p^length,
-// which is associative, so T is an inclusive scan of per-character pairs
-// (X[j] + 1, p).  Each CTA owns a tile of TILE_CHARS characters: a thread
-// folds 16 characters with Horner's rule, the CTA scans the 256 thread pairs
-// in shared memory, and tiles chain through a decoupled look-back on tile
-// descriptors (aggregate first, inclusive prefix when known), with tile ids
-// handed out in launch order by an atomic counter.  Reads 1 byte and writes
-// 8 bytes per character; with an output stride b > 1 it writes only the
-// prefixes of whole blocks, T[j] = h(X[0..jb)), the blocked table of
-// Sec. 3.3 (Alg. 2), 8/b bytes per character.
-#include <cstddef>
+//   h([S1, S2]) = h(S1) * p^|S2| + h(S2),
+// so T is a scan; all segments but the last have fixed lengths, so that only
+// hashes are scanned and every power is known beforehand.  Three passes: the
+// hashes of tiles of TILE_CHARS characters (16 characters a thread and row:
+// their codes times the split powers, summed in 64 bits and reduced once), one
+// CTA's scan of those (8 bytes per 16 KiB), and the output, in which each
+// thread extends its prefix over its characters.  The characters are read
+// twice, which costs a ninth of the output's traffic and saves every wait
+// between tiles: a single pass with a look-back chain spent two thirds of its
+// cycles at the barrier behind it (480 us for 10^8 characters).
+//
+// Reads 1 byte (twice) and writes 8 bytes per character, through shared memory
+// in whole lines; with an output stride b > 1 it writes only the prefixes of
+// whole blocks, T[j] = h(X[0..jb)), the blocked table of Sec. 3.3 (Alg. 2),
+// 8/b bytes per character.
+//
+// Bound: the bytes, and one modular product per character for its output
+// (about 35 instructions in all).  The first form took three products per
+// character and wrote at a 128-byte stride: 1057 us for 10^8 characters,
+// 370 us now (2430 GB/s of the 9 bytes a character).
+#include <algorithm>
 
 #include "ed_device.cuh"
 #include "lv_kernels.cuh"
 
 namespace edg {
 
-constexpr int HT = 256;                 // threads per scan CTA
-constexpr int HITEMS = 16;              // characters per thread
-constexpr int TILE_CHARS = HT * HITEMS; // 4096
-
-struct TileDesc {
-    unsigned long long agg_h, agg_p; // the tile's own pair
-    unsigned long long inc_h, inc_p; // pair of X[0 .. tile end)
-    uint32_t flag;                   // 0 none, 1 aggregate, 2 inclusive
-    uint32_t pad[3];
-};
-
-struct ScanState {
-    uint32_t next_tile;
-    uint32_t error;
-    uint32_t pad[14];
-    // TileDesc tiles[] follows (64-byte header)
-};
+constexpr int HT = 256;                 // threads per CTA
+constexpr int HW = HT / 32;             // its warps
+constexpr int HITEMS = 16;              // characters hashed, and written, at a time
+constexpr int HPARTS = 2;               // such parts a thread holds of a row
+constexpr int THREAD_CHARS = HPARTS * HITEMS;
+constexpr int ROW_CHARS = HT * THREAD_CHARS; // 8192
+constexpr int HROWS = 2;                // rows per tile
+constexpr int TILE_CHARS = HROWS * ROW_CHARS;
+constexpr int HPAD = HITEMS + 1;        // words between threads' outputs in shared memory
+constexpr int HPER_SM = 4;              // CTAs per SM (64 registers a thread, 35 KB each)
+constexpr int ST = 1024;                // threads of the tiles' scan
 
 size_t prefix_hash_state_bytes(int64_t len)
 {
     const int64_t tiles = (len + TILE_CHARS - 1) / TILE_CHARS + 1;
-    return 64 + sizeof(TileDesc) * (size_t)tiles;
+    return 2 * sizeof(uint64_t) * (size_t)tiles; // each tile's hash, and the prefix before it
 }
 
-struct HPair {
-    uint64_t h, p;
+// A multiplier b as mul61 takes it: b and b * 2^32 mod q, each hi * 2^31 + lo.
+struct Mul61 {
+    uint32_t c0l, c0h, c1l, c1h;
 };
-__device__ __forceinline__ HPair hcat(HPair a, HPair b)
+
+// The powers a launch uses.
+struct HashPowers {
+    uint32_t lo[HITEMS], hi[HITEMS]; // p^k = hi * 2^31 + lo, k < 16
+    uint64_t ones;                   // the hash of 16 characters of code 0, plus 1 each
+    Mul61 base;                      // p
+    Mul61 pow16[11];                 // p^(16 * 2^k): up to p^TILE_CHARS
+};
+
+// a * b mod q, below 2^62 + 2^34 (not reduced further), for a < 2^63: with
+// a = a1 2^32 + a0 it is a0 b + a1 (b 2^32), both split at 31 bits; 2^61 = 1.
+__device__ __forceinline__ uint64_t mul61(uint64_t a, const Mul61 &b)
 {
-    return {addmod61(mulmod61(a.h, b.p), b.h), mulmod61(a.p, b.p)};
+    const uint32_t a0 = (uint32_t)a, a1 = (uint32_t)(a >> 32);
+    const uint64_t sl = (uint64_t)a0 * b.c0l + (uint64_t)a1 * b.c1l; // < 2^63 + 2^62
+    const uint64_t sh = (uint64_t)a0 * b.c0h + (uint64_t)a1 * b.c1h; // < 2^62 + 2^61
+    return (sl & Q61) + (sl >> 61) + (sh >> 30) + ((sh & 0x3fffffffull) << 31);
+}
+__device__ __forceinline__ uint64_t fold61(uint64_t r) { return (r & Q61) + (r >> 61); } // below 2^61 + 8
+__device__ __forceinline__ uint64_t canon61(uint64_t r) // the residue below q, for r < 2^64
+{
+    r = (r & Q61) + (r >> 61);
+    return r >= Q61 ? r - Q61 : r;
+}
+__device__ __forceinline__ Mul61 mul_of(uint64_t b) // b < q
+{
+    // b * 2^32 mod q: b's upper 32 bits pass 2^61
+    const uint64_t c1 = canon61(((b << 32) & Q61) + (b >> 29));
+    return Mul61{(uint32_t)b & 0x7fffffffu, (uint32_t)(b >> 31), (uint32_t)c1 & 0x7fffffffu, (uint32_t)(c1 >> 31)};
 }
 
-__global__ void __launch_bounds__(HT) prefix_hash_kernel(const uint8_t *X, int64_t len, uint64_t base,
-                                                         uint64_t *T, int64_t stride,
-                                                         ScanState *st, uint64_t spin_ns)
+__device__ __forceinline__ uint32_t code_at(const uint4 &v, int i) // character i of 16
 {
-    __shared__ HPair s_pair[HT];
-    __shared__ HPair s_prefix;
-    __shared__ uint32_t s_tile;
-    TileDesc *tiles = reinterpret_cast<TileDesc *>(reinterpret_cast<unsigned char *>(st) + 64);
-    const int tid = threadIdx.x;
-    if (tid == 0)
-        s_tile = atomicAdd(&st->next_tile, 1u);
+    const uint32_t w = i < 4 ? v.x : (i < 8 ? v.y : (i < 12 ? v.z : v.w));
+    return __byte_perm(w, 0, 0x4440 + (i & 3));
+}
+
+// The hash of 16 characters, below 2^61 + 8.
+__device__ __forceinline__ uint64_t hash16(const HashPowers &P, const uint4 &v)
+{
+    uint64_t lo = 0, hi = 0; // below 2^45
+#pragma unroll
+    for (int i = 0; i < HITEMS; i++) {
+        const uint32_t c = code_at(v, i);
+        lo += (uint64_t)c * P.lo[HITEMS - 1 - i];
+        hi += (uint64_t)c * P.hi[HITEMS - 1 - i];
+    }
+    return fold61(lo + ((hi & 0x3fffffffull) << 31) + (hi >> 30) + P.ones);
+}
+// ... and of a thread's 32.
+__device__ __forceinline__ uint64_t hash32(const HashPowers &P, const uint4 (&v)[HPARTS])
+{
+    return fold61(mul61(hash16(P, v[0]), P.pow16[0]) + hash16(P, v[1]));
+}
+
+// The hash of every whole tile (one CTA each).
+__global__ void __launch_bounds__(HT) tile_hash_kernel(const uint8_t *X, int64_t len, uint64_t *agg,
+                                                       const __grid_constant__ HashPowers P)
+{
+    __shared__ uint64_t s_warp[HW];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t s0 = blockIdx.x * (int64_t)TILE_CHARS + (int64_t)tid * THREAD_CHARS;
+    uint4 v[HROWS][HPARTS];
+#pragma unroll
+    for (int r = 0; r < HROWS; r++)
+#pragma unroll
+        for (int q = 0; q < HPARTS; q++)
+            v[r][q] = load16(X, len, s0 + r * ROW_CHARS + q * HITEMS);
+    uint64_t h = 0;
+#pragma unroll
+    for (int r = 0; r < HROWS; r++)
+        h = fold61(mul61(h, P.pow16[9]) + hash32(P, v[r]));
+    // the threads' hashes (32 characters of each row) left to right
+#pragma unroll
+    for (int k = 0; k < 5; k++) {
+        const uint64_t o = __shfl_down_sync(0xffffffffu, h, 1 << k);
+        h = fold61(mul61(h, P.pow16[1 + k]) + o);
+    }
+    if (lane == 0)
+        s_warp[warp] = h;
     __syncthreads();
-    const int64_t tile = s_tile;
-    const int64_t t0 = tile * TILE_CHARS;
-    if (t0 >= len && !(len == 0 && tile == 0))
-        return;
-    // 1. this thread's 16 characters, folded with Horner's rule
-    const int64_t s0 = t0 + (int64_t)tid * HITEMS;
-    uint8_t c[HITEMS];
-    int cnt = 0;
-    if (s0 + HITEMS <= len && ((((uintptr_t)(X + s0)) & 15) == 0)) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(X + s0));
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    if (tid < 32) {
+        h = tid < HW ? s_warp[tid] : 0ull;
 #pragma unroll
-        for (int i = 0; i < HITEMS; i++)
-            c[i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
-        cnt = HITEMS;
-    } else {
-#pragma unroll
-        for (int i = 0; i < HITEMS; i++) {
-            const int64_t j = s0 + i;
-            c[i] = j < len ? __ldg(X + j) : 0;
+        for (int k = 0; k < 3; k++) {
+            const uint64_t o = __shfl_down_sync(0xffffffffu, h, 1 << k);
+            h = fold61(mul61(h, P.pow16[6 + k]) + o);
         }
-        cnt = (int)max((int64_t)0, min((int64_t)HITEMS, len - s0));
+        if (tid == 0)
+            agg[blockIdx.x] = canon61(h);
     }
-    HPair mine = {0, 1};
-    for (int i = 0; i < cnt; i++) {
-        mine.h = addmod61(mulmod61(mine.h, base), (uint64_t)c[i] + 1);
-        mine.p = mulmod61(mine.p, base);
+}
+
+// pre[t] = the hash of everything before tile t, t = 0 .. cnt, from the hashes
+// of tiles 0 .. cnt-1.  One CTA: every thread takes `per` consecutive tiles.
+__global__ void __launch_bounds__(ST) tile_scan_kernel(const uint64_t *agg, uint64_t *pre, int64_t cnt, int per,
+                                                       const __grid_constant__ HashPowers P)
+{
+    __shared__ uint64_t s_warp[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const Mul61 &tile = P.pow16[10];
+    const int64_t t0 = (int64_t)tid * per;
+    uint64_t h = 0, step = 1; // this thread's tiles; p^(TILE_CHARS * per)
+    for (int i = 0; i < per; i++) {
+        h = mul61(h, tile) + (t0 + i < cnt ? agg[t0 + i] : 0ull);
+        step = mul61(step, tile);
     }
-    // 2. inclusive scan of the thread pairs across the CTA (Hillis-Steele)
-    s_pair[tid] = mine;
+    h = canon61(h);
+    step = canon61(step);
+    uint64_t over = 1; // p^(TILE_CHARS * per * lane)
+#pragma unroll
+    for (int k = 0; k < 5; k++) {
+        const uint64_t o = __shfl_up_sync(0xffffffffu, h, 1 << k);
+        const Mul61 ms = mul_of(step);
+        if (lane >= 1 << k)
+            h = canon61(mul61(o, ms) + h);
+        if ((lane >> k) & 1)
+            over = canon61(mul61(over, ms));
+        step = canon61(mul61(step, ms));
+    }
+    if (lane == 31)
+        s_warp[warp] = h;
+    uint64_t excl = __shfl_up_sync(0xffffffffu, h, 1);
+    if (lane == 0)
+        excl = 0;
     __syncthreads();
-    for (int off = 1; off < HT; off <<= 1) {
-        HPair v = s_pair[tid];
-        if (tid >= off)
-            v = hcat(s_pair[tid - off], v);
-        __syncthreads();
-        s_pair[tid] = v;
-        __syncthreads();
+    if (warp == 0) {
+        uint64_t w = s_warp[lane];
+#pragma unroll
+        for (int k = 0; k < 5; k++) {
+            const uint64_t o = __shfl_up_sync(0xffffffffu, w, 1 << k);
+            const Mul61 ms = mul_of(step);
+            if (lane >= 1 << k)
+                w = canon61(mul61(o, ms) + w);
+            step = canon61(mul61(step, ms));
+        }
+        const uint64_t wx = __shfl_up_sync(0xffffffffu, w, 1);
+        s_warp[lane] = lane > 0 ? wx : 0ull;
     }
-    const HPair tile_agg = s_pair[HT - 1];
-    // 3. decoupled look-back for the prefix of everything before this tile
-    if (tid == 0) {
-        TileDesc &me = tiles[tile];
-        HPair prefix = {0, 1};
-        if (tile == 0) {
-            __stcg(&me.inc_h, tile_agg.h);
-            __stcg(&me.inc_p, tile_agg.p);
-            __threadfence();
-            st_release(&me.flag, 2u);
-        } else {
-            __stcg(&me.agg_h, tile_agg.h);
-            __stcg(&me.agg_p, tile_agg.p);
-            __threadfence();
-            st_release(&me.flag, 1u);
-            HPair run = {0, 1}; // pair of tiles (j, tile) exclusive, built right to left
-            int64_t j = tile - 1;
-            const uint64_t tstart = gtimer();
-            for (;;) {
-                uint32_t f;
-                while ((f = ld_acquire(&tiles[j].flag)) == 0) {
-                    if (gtimer() - tstart > spin_ns) {
-                        atomicCAS(&st->error, 0u, ST_TIMEOUT);
-                        break;
+    __syncthreads();
+    // what is before this thread's first tile: the warps before, carried over
+    // the lanes before, and those lanes
+    uint64_t t = canon61(mul61(s_warp[warp], mul_of(over)) + excl);
+    for (int i = 0; i < per; i++) {
+        if (t0 + i <= cnt)
+            pre[t0 + i] = t;
+        t = canon61(mul61(t, tile) + (t0 + i < cnt ? agg[t0 + i] : 0ull));
+    }
+}
+
+__global__ void __launch_bounds__(HT, HPER_SM) prefix_hash_kernel(const uint8_t *X, int64_t len, uint64_t *T,
+                                                                  int64_t stride, const uint64_t *pre,
+                                                                  const __grid_constant__ HashPowers P)
+{
+    __shared__ uint64_t s_out[HT * HPAD];
+    __shared__ uint64_t s_warp[2][HW];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t t0 = blockIdx.x * (int64_t)TILE_CHARS;
+    uint64_t before = pre ? pre[blockIdx.x] : 0ull; // everything before the row
+    if (blockIdx.x == 0 && tid == 0)
+        T[0] = 0;
+    // p^(32 lane), and the power that carries warp `lane`'s hash to the end of
+    // the row: p^(1024 (7 - lane))
+    uint64_t pl = 1, pe = 1;
+#pragma unroll
+    for (int k = 0; k < 5; k++)
+        if ((lane >> k) & 1)
+            pl = canon61(mul61(pl, P.pow16[1 + k]));
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+        if (((HW - 1 - lane) >> k) & 1)
+            pe = canon61(mul61(pe, P.pow16[6 + k]));
+    const Mul61 mlane = mul_of(pl), mend = mul_of(pe);
+    for (int r = 0; r < HROWS; r++) {
+        const int64_t r0 = t0 + r * ROW_CHARS;
+        if (r0 >= len)
+            break;
+        // 1. this thread's 32 characters and their hash (a thread with fewer
+        // ends the string: no thread reads its hash)
+        const int64_t s0 = r0 + (int64_t)tid * THREAD_CHARS;
+        uint4 v[HPARTS];
+#pragma unroll
+        for (int q = 0; q < HPARTS; q++)
+            v[q] = s0 + q * HITEMS < len ? load16(X, len, s0 + q * HITEMS) : make_uint4(0u, 0u, 0u, 0u);
+        // 2. inclusive scan across the warp, then every warp its own prefix
+        uint64_t h = hash32(P, v);
+#pragma unroll
+        for (int k = 0; k < 5; k++) {
+            const uint64_t o = __shfl_up_sync(0xffffffffu, h, 1 << k);
+            if (lane >= 1 << k)
+                h = fold61(mul61(o, P.pow16[1 + k]) + h);
+        }
+        if (lane == 31)
+            s_warp[r & 1][warp] = h;
+        uint64_t excl = __shfl_up_sync(0xffffffffu, h, 1);
+        if (lane == 0)
+            excl = 0;
+        __syncthreads(); // (also: the last row's outputs have been read)
+        uint64_t w = before; // everything before the warp
+        for (int q = 0; q < warp; q++)
+            w = fold61(mul61(w, P.pow16[6]) + s_warp[r & 1][q]);
+        // everything before the next row: the warps' hashes carried to the
+        // row's end, summed over lanes 0 .. 7
+        if (r + 1 < HROWS) {
+            uint64_t e = lane < HW ? fold61(mul61(s_warp[r & 1][lane], mend)) : 0ull;
+#pragma unroll
+            for (int o = 4; o; o >>= 1)
+                e += __shfl_xor_sync(0xffffffffu, e, o);
+            before = fold61(mul61(before, P.pow16[9]) + fold61(__shfl_sync(0xffffffffu, e, 0)));
+        }
+        // ... and before this thread
+        uint64_t t = mul61(w, mlane) + excl;
+        // 3. T for each character
+        if (stride == 1) {
+#pragma unroll
+            for (int q = 0; q < HPARTS; q++) {
+#pragma unroll
+                for (int i = 0; i < HITEMS; i++) {
+                    t = mul61(t, P.base) + code_at(v[q], i) + 1u;
+                    s_out[tid * HPAD + i] = canon61(t);
+                }
+                __syncthreads();
+                const int64_t q0 = r0 + q * HITEMS;
+                if (r0 + ROW_CHARS <= len) {
+#pragma unroll 8
+                    for (int i = 0; i < HITEMS; i++) {
+                        const int e = i * HT + tid, u = e / HITEMS, j = e % HITEMS;
+                        T[q0 + u * THREAD_CHARS + j + 1] = s_out[u * HPAD + j];
+                    }
+                } else {
+                    for (int e = tid; e < HT * HITEMS; e += HT) {
+                        const int u = e / HITEMS, j = e % HITEMS;
+                        if (q0 + u * THREAD_CHARS + j < len)
+                            T[q0 + u * THREAD_CHARS + j + 1] = s_out[u * HPAD + j];
                     }
                 }
-                if (f == 0) {
-                    prefix = {0, 1};
-                    break;
-                }
-                if (f == 2) {
-                    const HPair inc = {__ldcg(&tiles[j].inc_h), __ldcg(&tiles[j].inc_p)};
-                    prefix = hcat(inc, run);
-                    break;
-                }
-                const HPair agg = {__ldcg(&tiles[j].agg_h), __ldcg(&tiles[j].agg_p)};
-                run = hcat(agg, run);
-                j--;
+                __syncthreads();
             }
-            const HPair inc = hcat(prefix, tile_agg);
-            __stcg(&me.inc_h, inc.h);
-            __stcg(&me.inc_p, inc.p);
-            __threadfence();
-            st_release(&me.flag, 2u);
-        }
-        s_prefix = prefix;
-    }
-    __syncthreads();
-    // 4. the exclusive prefix of this thread's segment, then T for each char
-    HPair excl = s_prefix;
-    if (tid > 0)
-        excl = hcat(excl, s_pair[tid - 1]);
-    uint64_t h = excl.h;
-    if (tile == 0 && tid == 0)
-        T[0] = 0;
-    if (stride == 1) {
-        for (int i = 0; i < cnt; i++) {
-            h = addmod61(mulmod61(h, base), (uint64_t)c[i] + 1);
-            T[s0 + i + 1] = h;
-        }
-    } else {
-        // only the prefixes that end a whole block
-        int64_t next = (s0 / stride + 1) * stride; // first block end after s0
-        for (int i = 0; i < cnt; i++) {
-            h = addmod61(mulmod61(h, base), (uint64_t)c[i] + 1);
-            if (s0 + i + 1 == next) {
-                T[next / stride] = h;
-                next += stride;
+        } else {
+            // only the prefixes that end a whole block
+            int64_t next = (s0 / stride + 1) * stride; // first block end after s0
+#pragma unroll
+            for (int i = 0; i < THREAD_CHARS; i++) {
+                t = mul61(t, P.base) + code_at(v[i / HITEMS], i % HITEMS) + 1u;
+                if (s0 + i + 1 == next && next <= len) {
+                    T[next / stride] = canon61(t);
+                    next += stride;
+                }
             }
         }
     }
-
-}
-
-uint32_t prefix_hash_status(const void *scan_state, cudaStream_t s, cudaError_t *e)
-{
-    // the scan's status word (ST_TIMEOUT when a look-back wait gave up and
-    // the table after that tile is wrong), copied to the host stack
-    uint32_t st = 0;
-    *e = cudaMemcpyAsync(&st, static_cast<const unsigned char *>(scan_state) + offsetof(ScanState, error),
-                         sizeof(st), cudaMemcpyDeviceToHost, s);
-    if (*e == cudaSuccess)
-        *e = cudaStreamSynchronize(s);
-    return st;
 }
 
 cudaError_t launch_prefix_hash(const uint8_t *X, int64_t len, uint64_t base, uint64_t *T, int64_t stride,
-                               void *scan_state, size_t scan_state_bytes, cudaStream_t s)
+                               void *scan_state, cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(scan_state, 0, scan_state_bytes, s);
-    if (e != cudaSuccess)
-        return e;
     const int64_t tiles = len == 0 ? 1 : (len + TILE_CHARS - 1) / TILE_CHARS;
-    prefix_hash_kernel<<<(unsigned)tiles, HT, 0, s>>>(X, len, base, T, stride < 1 ? 1 : stride,
-                                                      reinterpret_cast<ScanState *>(scan_state),
-                                                      2000000000ull);
+    // the powers, by exact 128-bit products
+    auto mul = [](uint64_t x, uint64_t y) {
+        const unsigned __int128 z = (unsigned __int128)x * y;
+        uint64_t r = (uint64_t)(z & Q61) + (uint64_t)(z >> 61);
+        return r >= Q61 ? r - Q61 : r;
+    };
+    auto split = [&](uint64_t x) {
+        const uint64_t y = mul(x, 1ull << 32);
+        return Mul61{(uint32_t)(x & 0x7fffffffu), (uint32_t)(x >> 31), (uint32_t)(y & 0x7fffffffu), (uint32_t)(y >> 31)};
+    };
+    HashPowers P;
+    P.base = split(base);
+    uint64_t pw = 1;
+    for (int k = 0; k < HITEMS; k++, pw = mul(pw, base)) {
+        P.lo[k] = (uint32_t)(pw & 0x7fffffffu);
+        P.hi[k] = (uint32_t)(pw >> 31);
+        P.ones = (k ? P.ones : 0) + pw;
+        P.ones = P.ones >= Q61 ? P.ones - Q61 : P.ones;
+    }
+    for (int k = 0; k < 11; k++, pw = mul(pw, pw))
+        P.pow16[k] = split(pw);
+    uint64_t *agg = static_cast<uint64_t *>(scan_state), *pre = agg + tiles;
+    if (tiles > 1) { // (the last tile's hash is not needed)
+        tile_hash_kernel<<<(unsigned)(tiles - 1), HT, 0, s>>>(X, len, agg, P);
+        tile_scan_kernel<<<1, ST, 0, s>>>(agg, pre, tiles - 1, (int)((tiles + ST - 1) / ST), P);
+    }
+    prefix_hash_kernel<<<(unsigned)tiles, HT, 0, s>>>(X, len, T, stride < 1 ? 1 : stride, tiles > 1 ? pre : nullptr,
+                                                      P);
     return cudaGetLastError();
 }
 
@@ -208,7 +345,7 @@ cudaError_t launch_prefix_hash(const uint8_t *X, int64_t len, uint64_t base, uin
 // ---------------------------------------------------------------------------
 // Allocation-free prefix hash (see ed_prefix_hash_noalloc in include/ed.h).
 //
-// The scan's look-back descriptors live in this file-scope device array
+// The tiles' hashes and prefixes live in this file-scope device array
 // instead of memory the caller or a context allocates.  Every GPU that loads
 // the library holds it until the process exits.  Host code only ever uses
 // the array's device address, obtained once per device with
@@ -234,9 +371,9 @@ extern "C" int ed_prefix_hash_noalloc(const uint8_t *X, size_t len, uint64_t bas
 {
     if (!T || (len && !X) || base < 2 || base >= ((1ull << 61) - 1))
         return ED_EINVAL;
-    const size_t need = edg::prefix_hash_state_bytes((int64_t)len);
-    if (len > (size_t)INT64_MAX || need > NOALLOC_SCRATCH_BYTES)
-        return ED_EINVAL; // beyond the fixed scratch: at most ED_NOALLOC_MAX_LEN bytes
+    if (len > ED_NOALLOC_MAX_LEN)
+        return ED_EINVAL;
+    static_assert((ED_NOALLOC_MAX_LEN / edg::TILE_CHARS + 2) * 16 <= NOALLOC_SCRATCH_BYTES, "the tiles' words fit");
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= NOALLOC_MAX_DEVICES)
         return ED_ECUDA;
@@ -255,12 +392,7 @@ extern "C" int ed_prefix_hash_noalloc(const uint8_t *X, size_t len, uint64_t bas
         scratch = g_noalloc_addr[dev];
     }
     cudaStream_t s = (cudaStream_t)stream;
-    // the look-back descriptors must start at zero: cleared on every call
-    if (edg::launch_prefix_hash(X, (int64_t)len, base, T, 1, scratch, need, s) != cudaSuccess)
+    if (edg::launch_prefix_hash(X, (int64_t)len, base, T, 1, scratch, s) != cudaSuccess)
         return ED_ECUDA;
-    cudaError_t e = cudaSuccess;
-    const uint32_t st = edg::prefix_hash_status(scratch, s, &e);
-    if (e != cudaSuccess)
-        return ED_ECUDA;
-    return st == 0 ? ED_OK : (st == edg::ST_TIMEOUT ? ED_ETIMEOUT : ED_ECUDA);
+    return cudaStreamSynchronize(s) == cudaSuccess ? ED_OK : ED_ECUDA;
 }

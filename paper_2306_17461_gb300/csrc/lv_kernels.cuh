@@ -212,12 +212,9 @@ cudaError_t launch_lcp_queries(const uint8_t *A, int64_t n, const uint8_t *B, in
 // ---------------------------------------------------------------- hash
 // stride 1: T[i] = h(X[0..i)) for i = 0..len; stride b > 1: T[j] = h(X[0..jb))
 // for j = 0..len/b (the blocked table of Sec. 3.3)
+// scan_state: prefix_hash_state_bytes(len) of device memory, not cleared
 cudaError_t launch_prefix_hash(const uint8_t *X, int64_t len, uint64_t base, uint64_t *T, int64_t stride,
-                               void *scan_state, size_t scan_state_bytes, cudaStream_t s);
+                               void *scan_state, cudaStream_t s);
 size_t prefix_hash_state_bytes(int64_t len);
-// After a launch_prefix_hash on s: waits for s and returns the scan's status
-// word (0, or ST_TIMEOUT when a bounded look-back wait gave up); *e gets the
-// CUDA error of the copy or the wait.
-uint32_t prefix_hash_status(const void *scan_state, cudaStream_t s, cudaError_t *e);
 
 } // namespace edg

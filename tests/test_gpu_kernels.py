@@ -211,3 +211,23 @@ def test_confirmation_makes_wrong_hash_answers_exact(orc, blocked):
         assert reach.sum() > 20 and (wrong[reach] != want[reach]).mean() > 0.5  # the tables disagree
         got = ed.ed_lcp_dev(c1.h, dA, dB, xs, ys, confirmed, TA, TB)
         assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("stride", [1, 5])
+@pytest.mark.parametrize("length", [16_383, 16_384, 16_385, 24_577, 2 * 16_384 + 31, 1024 * 16_384 + 8_193])
+def test_prefix_hash_across_tiles(ctx, orc, length, stride):
+    """Lengths at the edges of a scan tile (16384 characters in two rows) and
+    past one tile per thread of the tiles' scan, from an unaligned start."""
+    from paper_2306_17461_gb300 import binding as ed
+
+    rng = np.random.default_rng(length + stride)
+    X = rng.integers(0, 256, length, dtype=np.uint8)
+    base = ed.ed_hash_base(ctx.h)
+    d = dev(np.concatenate([np.zeros(3, np.uint8), X]))[3:]
+    if stride == 1:
+        T = ed.ed_prefix_hash_dev(ctx.h, d)
+        want = orc.prefix_hash(X, base)
+    else:
+        T = ed.ed_prefix_hash_blocked_dev(ctx.h, d, stride)
+        want = orc.prefix_hash_blocked(X, stride, base)
+    assert np.array_equal(T.cpu().numpy().view(np.uint64), want)
