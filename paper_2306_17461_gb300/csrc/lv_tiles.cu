@@ -150,6 +150,55 @@ __device__ __noinline__ int64_t hash_lcp(const uint64_t *pow2, const HashView VA
     return good;
 }
 
+// The same search by a whole warp (identical arguments on every lane, the
+// answer on every lane): the doubling lengths tested at once, then the
+// bracket cut into 32 a step.  A probe waits on a round trip to the tables, so
+// that the chain of dependent probes bounds the query: about 5 here where one
+// thread takes 2 log2(l) (28 at l = 10^4; a query took 18 us of a round's 21).
+__device__ __noinline__ int64_t hash_lcp_warp(const uint64_t *pow2, const HashView VA, const HashView VB,
+                                              int64_t x, int64_t y, int64_t lim)
+{
+    const int lane = threadIdx.x & 31;
+    const uint64_t p = pow2[0];
+    const uint64_t hx = prefix_at(VA, x, p), hy = prefix_at(VB, y, p);
+    auto equal = [&](int64_t L, uint64_t P) {
+        return submod61(prefix_at(VA, x + L, p), mulmod61(hx, P)) ==
+               submod61(prefix_at(VB, y + L, p), mulmod61(hy, P));
+    };
+    // 2^lane, where it is below lim; lim itself only when all of those agree
+    const int64_t L = 1ll << lane;
+    const bool in = lane < 31 && L < lim;
+    const unsigned int bad0 = __ballot_sync(0xffffffffu, in && !equal(L, pow2[lane]));
+    int64_t good, bad = lim;
+    int j = __popc(__ballot_sync(0xffffffffu, in)); // lengths 2^0 .. 2^(j-1) agree
+    if (bad0) {
+        j = __ffs((int)bad0) - 1;
+        bad = 1ll << j;
+    } else if (equal(lim, powp(pow2, lim))) {
+        return lim;
+    }
+    good = j ? 1ll << (j - 1) : 0;
+    uint64_t pg = j ? pow2[j - 1] : 1ull;
+    // the largest length in [good, bad) whose hashes agree, five bits a step
+    for (int k = 64 - __clzll((long long)(bad - good - 1)); k > 0;) {
+        const int step = max(k - 5, 0);
+        const int64_t cand = good + ((int64_t)lane << step);
+        uint64_t Pc = pg;
+#pragma unroll
+        for (int b = 0; b < 5; b++)
+            if ((lane >> b) & 1)
+                Pc = mulmod61(Pc, pow2[step + b]);
+        const bool agree = lane == 0 || (cand < bad && equal(cand, Pc));
+        const unsigned int fail = __ballot_sync(0xffffffffu, !agree);
+        const int f = fail ? __ffs((int)fail) - 1 : 32;
+        bad = min(bad, good + ((int64_t)f << step));
+        good += (int64_t)(f - 1) << step;
+        pg = __shfl_sync(0xffffffffu, Pc, f - 1);
+        k = step;
+    }
+    return good;
+}
+
 // ------------------------------------------------------------------ pair
 struct Pair {
     const uint8_t *A, *B;
@@ -953,16 +1002,17 @@ __device__ __forceinline__ unsigned long long *halo_ptr(const LvArgs &P, int cta
 }
 
 // The bound of an open slide of diagonal d from row c: the string end, or
-// the hash answer + 1 (the slide confirms it directly).
+// the hash answer + 1 (the slide confirms it directly).  A whole warp calls it.
 __device__ __forceinline__ int64_t open_limit(const LvArgs &P, const Pair &Q, int64_t c, int64_t d, Counters &C,
                                               bool own)
 {
     const int64_t full = min(Q.n - c, Q.m - c - d);
     int64_t lim = full;
     if (Q.hash && full > 0) {
-        const int64_t h = hash_lcp(P.pow2, HashView{Q.TA, Q.A, P.hash_b}, HashView{Q.TB, Q.B, P.hash_b}, c,
-                                   c + d, 0, full);
-        C.hashq += own;
+        const int64_t h = hash_lcp_warp(P.pow2, HashView{Q.TA, Q.A, P.hash_b}, HashView{Q.TB, Q.B, P.hash_b}, c,
+                                        c + d, full);
+        if ((threadIdx.x & 31) == 0)
+            C.hashq += own;
         lim = min(h + 1, full);
     }
     return c + lim;
@@ -986,12 +1036,9 @@ __device__ __forceinline__ void warp_slides(const LvArgs &P, const Pair &Q, int3
     for (int j = w0; j < nl; j += ws) {
         const int64_t d = Ld[j], c = Lc[j];
         const bool own = d >= a && d < b;
-        int64_t lim = 0;
-        if (lane == 0) {
-            lim = open_limit(P, Q, c, d, C, own);
+        const int64_t lim = open_limit(P, Q, c, d, C, own);
+        if (lane == 0)
             C.opens += own;
-        }
-        lim = __shfl_sync(0xffffffffu, lim, 0);
         bool open;
         const int64_t l = slide_warp(Q.A, Q.n, Q.B, Q.m, c, c + d, 0, lim - c, P.t2_cap, &open);
         if (!open && l >= PREFETCH_MIN) // a long slide: the next round starts past it
@@ -1039,8 +1086,11 @@ __device__ __forceinline__ void cta_slides(const LvArgs &P, const Smem S, const 
         any = true;
         const int64_t c = Lc[j];
         const bool own = d >= a && d < b;
-        if (tid == 0)
-            S.bcl[3] = open_limit(P, Q, c, d, C, false);
+        if (tid < 32) {
+            const int64_t l = open_limit(P, Q, c, d, C, false);
+            if (tid == 0)
+                S.bcl[3] = l;
+        }
         __syncthreads();
         const int64_t lim = S.bcl[3];
         __syncthreads();
