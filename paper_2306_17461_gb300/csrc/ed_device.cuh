@@ -517,6 +517,109 @@ __device__ __forceinline__ int64_t sweep_scan(const uint8_t *A, int64_t n, const
     return -1;
 }
 
+// The calling CTA compares A[x0 .. x0+len) with B[y0 ..) for any len (x0 +
+// len <= n, y0 + len <= m), blockDim.x * 16 * U bytes of each string a step
+// (32 KiB at 256 threads, U = 8), the next step's loads in flight while one
+// is compared: the blocks of sweep_scan, kept in registers.  Returns the first
+// mismatching offset, or -1.  One SM draws about 64 bytes a cycle: 10^4 bytes
+// take 2 to 3 thousand cycles, 10^5 about 6 thousand (opening them to other
+// CTAs takes 14 thousand and more).  Every thread must call it.
+template <int U>
+struct SweepStep {
+    uint4 a[U], b[U], x;
+};
+template <int U>
+__device__ __forceinline__ void sweep_load(SweepStep<U> &s, uintptr_t A, int64_t n, uintptr_t B, int64_t m,
+                                           uintptr_t a0, uintptr_t b0, int64_t j0)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+        s.a[u] = ld_stream16(safe_blk(A, n, a0 + 16 * (j0 + u * 32 + lane)));
+        s.b[u] = ld_stream16(safe_blk(B, m, b0 + 16 * (j0 + u * 32 + lane)));
+    }
+    s.x = ld_stream16(safe_blk(B, m, b0 + 16 * (j0 + 32 * U)));
+}
+// The first mismatching offset of the thread's blocks, or -1.
+template <int U>
+__device__ __forceinline__ int64_t sweep_compare(const SweepStep<U> &s, uint32_t sa, uint32_t qb, int64_t j0,
+                                                 int64_t len)
+{
+    const int lane = threadIdx.x & 31;
+    int64_t best = -1;
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+        const uint4 nb = u + 1 < U ? s.b[u + 1 < U ? u + 1 : 0] : s.x;
+        uint4 nx; // the B block after this lane's
+        nx.x = __shfl_sync(0xffffffffu, lane == 0 ? nb.x : s.b[u].x, (lane + 1) & 31);
+        nx.y = __shfl_sync(0xffffffffu, lane == 0 ? nb.y : s.b[u].y, (lane + 1) & 31);
+        nx.z = __shfl_sync(0xffffffffu, lane == 0 ? nb.z : s.b[u].z, (lane + 1) & 31);
+        nx.w = __shfl_sync(0xffffffffu, lane == 0 ? nb.w : s.b[u].w, (lane + 1) & 31);
+        const uint4 bs = shift_bytes(s.b[u], nx, qb);
+        if (best < 0 && ((s.a[u].x ^ bs.x) | (s.a[u].y ^ bs.y) | (s.a[u].z ^ bs.z) | (s.a[u].w ^ bs.w))) {
+            // the first differing byte inside [0, len): offsets o0 + i
+            const int64_t o0 = 16 * (j0 + u * 32 + lane) - (int64_t)sa;
+            uint64_t d0 = ((uint64_t)(s.a[u].y ^ bs.y) << 32) | (s.a[u].x ^ bs.x);
+            uint64_t d1 = ((uint64_t)(s.a[u].w ^ bs.w) << 32) | (s.a[u].z ^ bs.z);
+            if (o0 < 0) { // (only the first block: sa bytes before the start)
+                const int skip = (int)-o0;
+                d0 &= skip >= 8 ? 0ull : ~0ull << (8 * skip);
+                d1 &= skip <= 8 ? ~0ull : ~0ull << (8 * (skip - 8));
+            }
+            int i = 16;
+            if (d0)
+                i = (__ffsll((long long)d0) - 1) >> 3;
+            else if (d1)
+                i = 8 + ((__ffsll((long long)d1) - 1) >> 3);
+            if (i < 16 && o0 + i < len)
+                best = o0 + i;
+        }
+    }
+    return best;
+}
+template <int U>
+__device__ __noinline__ int64_t stream_sweep(const uint8_t *A, int64_t n, const uint8_t *B, int64_t m, int64_t x0,
+                                             int64_t y0, int64_t len, unsigned long long *s_min)
+{
+    const uintptr_t pa = (uintptr_t)(A + x0), pb = (uintptr_t)(B + y0);
+    const uint32_t sa = (uint32_t)(pa & 15), qb = (uint32_t)((pb - sa) & 15);
+    const uintptr_t a0 = pa - sa, b0 = pb - sa - qb;
+    const uintptr_t Ab = (uintptr_t)A, Bb = (uintptr_t)B;
+    const int64_t nblk = ((int64_t)sa + len + 15) >> 4, step = (int64_t)(blockDim.x >> 5) * 32 * U;
+    int64_t j = (int64_t)(threadIdx.x >> 5) * 32 * U; // this warp's first block
+    if (threadIdx.x == 0)
+        *s_min = ~0ull;
+    SweepStep<U> s0, s1;
+    sweep_load(s0, Ab, n, Bb, m, a0, b0, j);
+    for (int64_t at = 0;;) {
+        // two steps a turn, so that each buffer stays in its registers
+        int64_t best;
+        const bool more1 = at + step < nblk;
+        if (more1)
+            sweep_load(s1, Ab, n, Bb, m, a0, b0, j + step);
+        best = sweep_compare(s0, sa, qb, j, len);
+        at += step;
+        j += step;
+        bool hit = __syncthreads_or(best >= 0) != 0;
+        if (!hit && more1) {
+            if (at + step < nblk)
+                sweep_load(s0, Ab, n, Bb, m, a0, b0, j + step);
+            best = sweep_compare(s1, sa, qb, j, len);
+            at += step;
+            j += step;
+            hit = __syncthreads_or(best >= 0) != 0;
+        }
+        if (hit) {
+            if (best >= 0)
+                atomicMin(s_min, (unsigned long long)best);
+            __syncthreads();
+            return (int64_t)*s_min; // (the caller meets a barrier before the next use)
+        }
+        if (at >= nblk)
+            return -1;
+    }
+}
+
 // ------------------------------------------------------- bulk copies
 // Shared-memory address of a generic pointer into shared memory.
 __device__ __forceinline__ uint32_t smem_u32(const void *p)

@@ -322,6 +322,7 @@ struct Smem {
     unsigned long long *smin;
     JobDesc *jd;        // the job last claimed from
     int *jring;         // the CTA's next job slot (0 .. JOB_RING-1)
+    int *run;           // mean length of its long slides (long_slide)
     unsigned char *stg; // bulk-copy staging of one chunk (null: none), see stage_of
     int lcap;
     uint32_t *err;             // launch status word (self-check records)
@@ -799,41 +800,40 @@ __device__ __noinline__ int64_t run_job(const LvArgs &P, const Smem S, const Pai
 }
 
 // The CTA's own long slide: the first mismatch of A[x..x+lim) vs B[y..).
-// The CTA scans the first local_chunks chunks alone (after one bulk L2
-// prefetch of all of them); the rest goes to jobs of at most JOB_MAX_CHUNKS
-// chunks each, helped by other CTAs.  Returns the first mismatch offset, or
-// lim.
+// *run is the running mean length of the CTA's long slides (on the alignment
+// path slides long and short come in runs).  While it is at most RUN_BYTES the
+// CTA streams up to ALONE_BYTES of each string itself (local_chunks chunks at
+// least); the rest, and the whole of a slide when they run longer, goes to
+// jobs of at most JOB_MAX_CHUNKS chunks each, helped by other CTAs.  A job
+// takes 14 to 20 thousand cycles however short its slide is; the CTA alone
+// takes 3 thousand for 10^4 bytes and as many as a job for about 10^5.
+// Returns the first mismatch offset, or lim (every thread; a barrier lies
+// between two calls).
+constexpr int64_t ALONE_BYTES = 64 * 1024;
+constexpr int RUN_BYTES = 32 * 1024;
 __device__ __noinline__ int64_t long_slide(const LvArgs &P, const Smem S, const Pair Q, int64_t x0,
                                            int64_t y0, int64_t lim0)
 {
-    const int tid = threadIdx.x;
-    const int64_t loc = min(lim0, (int64_t)max(0, P.local_chunks) * CHUNK_BYTES);
-    if (tid == 0 && loc > CHUNK_BYTES) {
-        bulk_prefetch_l2(Q.A, Q.n, x0 + CHUNK_BYTES, loc - CHUNK_BYTES);
-        bulk_prefetch_l2(Q.B, Q.m, y0 + CHUNK_BYTES, loc - CHUNK_BYTES);
-    }
-    int64_t off = 0;
-    if (S.stg && P.stage >= 2 && loc > CHUNK_BYTES) {
-        // the chunks in turn through two stages, the next one's copies in flight
-        const int64_t r = stream_scan<CHUNK_BYTES>(stage_of(S.stg), stage_of(S.stg + STAGE_STRIDE), Q.A, Q.n, Q.B,
-                                                   Q.m, x0, y0, loc, S.smin, P.spin_ns, S.err);
-        if (r < loc)
-            return r >= 0 ? r : lim0; // (-2: a wait gave up; the launch reports it)
-        off = loc;
-    }
-    for (; off < loc; off += CHUNK_BYTES) {
-        const int64_t r = chunk_scan(P, S, Q.A, Q.n, Q.B, Q.m, x0 + off, y0 + off, min((int64_t)CHUNK_BYTES, lim0 - off));
-        if (r >= 0)
-            return off + r;
-    }
-    while (off < lim0) {
+    const int mean = *S.run;
+    const int64_t loc = min(lim0, max(mean <= RUN_BYTES ? ALONE_BYTES : (int64_t)0,
+                                      (int64_t)max(0, P.local_chunks) * CHUNK_BYTES));
+    int64_t r = -1;
+    if (loc > 0)
+        r = stream_sweep<2>(Q.A, Q.n, Q.B, Q.m, x0, y0, loc, S.smin);
+    int64_t off = loc;
+    while (r < 0 && off < lim0) {
         const int64_t len = min(lim0 - off, (int64_t)JOB_MAX_CHUNKS * CHUNK_BYTES);
-        const int64_t r = run_job(P, S, Q, x0 + off, y0 + off, len);
-        if (r < len)
-            return off + r;
+        const int64_t q = run_job(P, S, Q, x0 + off, y0 + off, len);
+        if (q < len)
+            r = off + q;
         off += len;
     }
-    return lim0;
+    if (r < 0)
+        r = lim0;
+    __syncthreads(); // every thread has read *S.run and the sweep's answer
+    if (threadIdx.x == 0)
+        *S.run = mean + (((int)min(r, (int64_t)1 << 24) - mean) >> 2);
+    return r;
 }
 
 // ------------------------------------------------------------------ group
@@ -917,6 +917,7 @@ __device__ Smem carve(const LvArgs &P)
     S.nR = S.nL + 7;
     S.jd = reinterpret_cast<JobDesc *>(p + 192);
     S.jring = reinterpret_cast<int *>(p + 48);
+    S.run = reinterpret_cast<int *>(p + 72);
     // p + 176: lone (lean_slides); p + 184: the tile's lead at an epoch change
     p += 256;
     S.lcap = P.smax + 2 * HMAX + 2;
@@ -1095,8 +1096,7 @@ __device__ __forceinline__ void cta_slides(const LvArgs &P, const Smem S, const 
         const int64_t lim = S.bcl[3];
         __syncthreads();
         const int64_t rr = long_slide(P, S, Q, c, c + d, lim - c);
-        if (lim - c > (int64_t)max(0, P.local_chunks) * CHUNK_BYTES) // published as a job
-            C.longs++;
+        C.longs++;
         if (tid < 32)
             prefetch_next(Q.A, Q.n, Q.B, Q.m, c + rr, c + rr + d);
         if (tid == 0)
@@ -1291,10 +1291,13 @@ __device__ __forceinline__ BlockOut run_block(const LvArgs &P, const Smem S, con
     return BlockOut{C.slide, C.mism, C.hashq, C.coll, C.longs, C.opens, C.tm[0], C.tm[1], kfound >= 0 ? 1 : 0};
 }
 
+// A lone slide this long is worth the whole CTA (one step of stream_sweep).
+constexpr int32_t LONE_BYTES = 2048;
+
 // The open slides of a lean round (out of line: most rounds have none):
 // one warp each, up to t2_cap bytes, then the whole CTA for those still
-// open -- or, for a lone slide after a lone one that outran its warp, the
-// whole CTA at once.  Every thread calls it (after a barrier); the final
+// open -- or, for a lone slide after a lone one that outran its warp (or went
+// on for LONE_BYTES), the whole CTA at once.  Every thread calls it (after a barrier); the final
 // rows are visible to every thread when it returns.
 __device__ __forceinline__ void lean_slides(const LvArgs &P, const Smem S, const Pair Q, int32_t *cur, int64_t off,
                                          int32_t *Ld, const int32_t *Lc, int nlo, int64_t a, int64_t b, int pr,
@@ -1306,6 +1309,20 @@ __device__ __forceinline__ void lean_slides(const LvArgs &P, const Smem S, const
     // and short come in runs
     int *lone = reinterpret_cast<int *>(reinterpret_cast<unsigned char *>(S.jring) + 128);
     const bool direct = nlo == 1 && *lone != 0;
+    if (direct && !Q.hash) {
+        const int64_t d = Ld[0], c = Lc[0], lim = min(Q.n - c, Q.m - c - d);
+        const int64_t rr = long_slide(P, S, Q, c, c + d, lim);
+        C.longs++;
+        if (threadIdx.x < 32) {
+            if (threadIdx.x == 0) {
+                cur[d - off] = (int32_t)finish_slide(Q, c, d, c + rr, c + lim, d >= a && d < b, C);
+                *lone = rr > LONE_BYTES;
+            }
+            prefetch_next(Q.A, Q.n, Q.B, Q.m, c + rr, c + rr + d);
+        }
+        __syncthreads();
+        return;
+    }
     if (direct) {
         cta_slides(P, S, Q, cur, off, Ld, Lc, nlo, a, b, C);
     } else {
@@ -1317,7 +1334,7 @@ __device__ __forceinline__ void lean_slides(const LvArgs &P, const Smem S, const
     }
     if (threadIdx.x == 0) {
         if (nlo == 1)
-            *lone = direct ? (cur[Ld[0] - off] - Lc[0] > P.t2_cap) : S.left[pr];
+            *lone = direct ? (cur[Ld[0] - off] - Lc[0] > LONE_BYTES) : S.left[pr];
         S.left[pr] = 0;
     }
     __syncthreads();
@@ -1521,8 +1538,12 @@ __device__ __forceinline__ bool run_pair(const LvArgs &P, const Smem S, const Pa
         S.F0[i] = NEG;
         S.F1[i] = NEG;
     }
-    if (tid == 0)
+    if (tid == 0) {
         *S.n1 = 0;
+        // (nothing known yet: the first slide of a string of 8 MB and more is
+        // opened to other CTAs at once)
+        *S.run = (int)(min(n, m) >> 8);
+    }
     __syncthreads();
     if (t > 0 && T.has) {
         // round t - 1 of the tile and its halo from the keep buffer
