@@ -432,8 +432,8 @@ __device__ __forceinline__ uintptr_t safe_blk(uintptr_t base, int64_t len, uintp
 }
 
 // The calling CTA compares A[x0 .. x0+len) with B[y0 .. y0+len) for
-// len <= blockDim.x * 16 * U (32 KiB per string at 256 threads, U = 8) and
-// returns the first mismatching offset, or -1 if all are equal.  Needs
+// len <= blockDim.x * 16 * U - 16 (the blocks start up to 15 bytes before the
+// bytes compared) and returns the first mismatching offset, or -1.  Needs
 // x0 + len <= n and y0 + len <= m.  Every load is issued before the first
 // compare: one memory round trip per call.
 //
@@ -520,10 +520,10 @@ __device__ __forceinline__ int64_t sweep_scan(const uint8_t *A, int64_t n, const
 // The calling CTA compares A[x0 .. x0+len) with B[y0 ..) for any len (x0 +
 // len <= n, y0 + len <= m), blockDim.x * 16 * U bytes of each string a step
 // (32 KiB at 256 threads, U = 8), the next step's loads in flight while one
-// is compared: the blocks of sweep_scan, kept in registers.  Returns the first
-// mismatching offset, or -1.  One SM draws about 64 bytes a cycle: 10^4 bytes
-// take 2 to 3 thousand cycles, 10^5 about 6 thousand (opening them to other
-// CTAs takes 14 thousand and more).  Every thread must call it.
+// is compared, all in registers.  Returns the first mismatching offset, or -1.
+// The blocks are sweep_scan's.  10^4 bytes take about 3 thousand cycles.  Every
+// thread must call it; s_min is a shared 64-bit scratch word, and the caller
+// meets a barrier before the next use.
 template <int U>
 struct SweepStep {
     uint4 a[U], b[U], x;

@@ -56,13 +56,11 @@ constexpr int WATCH_SPINS = 8;
 constexpr int WATCH_WORDS = 4; // answer words a lane loads per look
 constexpr uint64_t OWN_SCAN_NS = 1000;
 
+// A thread's counts of the block of rounds (and then of the pair) in
+// progress; the times of its phases lie in shared memory (Smem::tm).
 struct Counters {
-    unsigned long long slide = 0, mism = 0, hashq = 0, coll = 0, longs = 0, blocks = 0, opens = 0;
-    unsigned long long tm[4] = {0, 0, 0, 0};
-};
-// What one call of open_slides adds to the counters.
-struct SlideCounts {
-    unsigned long long slide, mism, hashq, coll, longs, opens;
+    unsigned long long slide = 0, mism = 0;
+    uint32_t hashq = 0, coll = 0, longs = 0, blocks = 0, opens = 0;
 };
 
 // ------------------------------------------------------------------ hash
@@ -286,8 +284,14 @@ struct JobDesc {
     uint32_t jid;
     int32_t slot;
     int32_t pq; // the pair whose strings A, B are (-1: none yet)
+    int32_t chunk; // bytes of one claim
 };
-static_assert(sizeof(JobDesc) <= 64, "the job cache fills bytes 192..255 of the smem header");
+// The descriptor's pair word: the pair's index, and above it whether the job
+// goes in small chunks: one sweep of the CTA each, a 16-byte block a thread
+// (less the 15 bytes the blocks may start early).
+constexpr uint32_t PAIR_MASK = (1u << 31) - 1;
+constexpr int SMALL_CHUNK = CTA_THREADS * 16 - 16;
+__device__ __forceinline__ int32_t chunk_bytes(bool small) { return small ? SMALL_CHUNK : CHUNK_BYTES; }
 
 // Bytes between consecutive stages (128-byte aligned).
 constexpr size_t STAGE_STRIDE = (stage_bytes<CHUNK_BYTES>() + 127) & ~(size_t)127;
@@ -304,29 +308,53 @@ __device__ __forceinline__ Stage stage_of(unsigned char *p)
     return T;
 }
 
-// Kept in registers: every function takes it by value (no address taken,
-// no array member indexed at run time).
+// The CTA's shared memory.  Every part lies at an offset known at compile
+// time, or behind the frontier buffers (smax wide): the accessors cost no
+// register, where a struct of the twenty pointers took forty in every function
+// that calls another.
+extern __shared__ __align__(128) unsigned char tiles_raw[];
+constexpr int OCAP = 1024;     // open slides listed per round (pipelined rounds)
+constexpr int DCAP = 3 * OCAP; // deferred diagonals: neighbours of open ones
+constexpr int HEADER = 384;
 struct Smem {
-    int32_t *F0, *F1;   // tile + halo frontier, smax + 2*HMAX + 2 entries each
-    int32_t *ld;        // open slides: diagonal (lcap entries)
-    // pipelined rounds: open lists by round parity (diagonal, start row;
-    // OCAP entries each) and their counts, the deferred diagonals of a round
-    int32_t *Ld0, *Ld1, *Lc0, *Lc1, *D;
-    int *nL, *nD;       // by round parity
-    int *left;          // a slider warp left a listed slide open (by round parity)
-    int *kf;            // the target diagonal reached row n in the round before
-    int *nR;            // deferred diagonals a slider warp computed (by round parity)
-    int *n1;
-    int *bc;            // 8 broadcast words
-    long long *bcl;     // 4 broadcast 64-bit words
-    unsigned long long *smin;
-    JobDesc *jd;        // the job last claimed from
-    int *jring;         // the CTA's next job slot (0 .. JOB_RING-1)
-    int *run;           // mean length of its long slides (long_slide)
-    unsigned char *stg; // bulk-copy staging of one chunk (null: none), see stage_of
-    int lcap;
-    uint32_t *err;             // launch status word (self-check records)
-    unsigned long long *diag;
+    int32_t smax, stage;
+    template <typename T>
+    __device__ __forceinline__ static T *at(size_t o) { return reinterpret_cast<T *>(tiles_raw + o); }
+    __device__ __forceinline__ size_t wide() const { return sizeof(int32_t) * (size_t)(smax + 2 * HMAX + 2); }
+    __device__ __forceinline__ unsigned long long *smin() const { return at<unsigned long long>(0); }
+    __device__ __forceinline__ long long *bcl() const { return at<long long>(16); } // 4 broadcast 64-bit words
+    __device__ __forceinline__ int *jring() const { return at<int>(48); } // the CTA's next job slot (0 .. JOB_RING-1)
+    __device__ __forceinline__ int *n1() const { return at<int>(64); }
+    __device__ __forceinline__ int *run() const { return at<int>(72); } // mean length of its long slides (long_slide)
+    __device__ __forceinline__ int *bc() const { return at<int>(80); }  // 8 broadcast words
+    __device__ __forceinline__ int *jids() const { return at<int>(112); } // the job ids its slots have reached
+    // by round parity: open slides listed, deferred diagonals, a slide that
+    // outran its warp, deferred diagonals a slider warp computed
+    __device__ __forceinline__ int *nL() const { return at<int>(128); }
+    __device__ __forceinline__ int *nD() const { return at<int>(136); }
+    __device__ __forceinline__ int *left() const { return at<int>(144); }
+    __device__ __forceinline__ int *kf() const { return at<int>(152); } // the target row was n in the round before
+    __device__ __forceinline__ int *nR() const { return at<int>(156); }
+    __device__ __forceinline__ int *lone() const { return at<int>(176); } // lean_slides
+    __device__ __forceinline__ unsigned long long *lead() const { return at<unsigned long long>(184); }
+    __device__ __forceinline__ JobDesc *jd() const { return at<JobDesc>(192); } // the job last claimed from
+    // cycles in rounds, open slides, halo waits and epoch changes (thread 0's)
+    __device__ __forceinline__ unsigned long long *tm() const { return at<unsigned long long>(256); }
+    // tile + halo frontier by round parity, smax + 2*HMAX + 2 entries each
+    __device__ __forceinline__ int32_t *F0() const { return at<int32_t>(HEADER); }
+    __device__ __forceinline__ int32_t *F1() const { return at<int32_t>(HEADER + wide()); }
+    // open lists by round parity (diagonal, start row), the deferred diagonals
+    __device__ __forceinline__ int32_t *Ld0() const { return at<int32_t>(HEADER + 2 * wide()); }
+    __device__ __forceinline__ int32_t *Ld1() const { return Ld0() + OCAP; }
+    __device__ __forceinline__ int32_t *Lc0() const { return Ld0() + 2 * OCAP; }
+    __device__ __forceinline__ int32_t *Lc1() const { return Ld0() + 3 * OCAP; }
+    __device__ __forceinline__ int32_t *D() const { return Ld0() + 4 * OCAP; }
+    // bulk-copy staging of chunks (null: none), see stage_of
+    __device__ __forceinline__ unsigned char *stg() const
+    {
+        const size_t o = HEADER + 2 * wide() + sizeof(int32_t) * (4 * OCAP + DCAP);
+        return stage ? tiles_raw + ((o + 127) & ~(size_t)127) : nullptr;
+    }
 };
 
 // Job slot protocol.  claim = (job id << 32) | count: every atomicAdd of 1
@@ -336,9 +364,11 @@ struct Smem {
 // and the answers are raised by red.max, so an answer of a job the slot no
 // longer holds (from a claimer that fell behind) never overwrites one of the
 // job it holds.  A slot is therefore reused with no wait for the claims of
-// its last job, and nothing is cleared.  A claim that lands on a job
-// published after the claimer looked is a claim of that job (the descriptor
-// read after the atomic, and a fence, carries its id).
+// its last job, and nothing is cleared.  The owner publishes with plain
+// relaxed stores (a release waited 2 thousand cycles for them): a claimer
+// whose claim ran ahead of the descriptor sees an older job's id in it and
+// looks again.  A claim that lands on a job published after the claimer
+// looked is a claim of that job.
 //   ans[c]  = (jid << 32) | job offset of the chunk's first mismatch (NOMIS: none)
 //   result  = (jid << 32) | ~best  (so that red.max keeps the least offset)
 constexpr uint32_t NOMIS = 0xffffffffu;
@@ -383,7 +413,7 @@ __device__ __forceinline__ int claim_go(const LvArgs &P, const Smem S, JobSlot *
 {
     const uint32_t jid = (uint32_t)(w >> 32);
     const int64_t c = (int64_t)(uint32_t)w;
-    JobDesc *J = S.jd;
+    JobDesc *J = S.jd();
     if (J->jid != jid || J->slot != s) {
         // the words read along with the claim serve when they all carry its
         // job (each word holds its tag with its value); else read them again
@@ -398,28 +428,34 @@ __device__ __forceinline__ int claim_go(const LvArgs &P, const Smem S, JobSlot *
             tags = (uint32_t)(xt >> 32) == jid && (uint32_t)(yt >> 32) == jid && (uint32_t)(lt >> 32) == jid &&
                    (uint32_t)(pt >> 32) == jid;
         }
-        if (!tags) {
-            __threadfence();
+        for (int look = 0; !tags; look++) {
             xt = ld_relaxed_u64(&sl->xt);
             yt = ld_relaxed_u64(&sl->yt);
             lt = ld_relaxed_u64(&sl->lt);
             pt = ld_relaxed_u64(&sl->pt);
             best = ld_relaxed_u64(&sl->result);
-            if ((uint32_t)(xt >> 32) != jid || (uint32_t)(yt >> 32) != jid || (uint32_t)(lt >> 32) != jid ||
-                (uint32_t)(pt >> 32) != jid) {
+            const uint32_t t0 = (uint32_t)(xt >> 32), t1 = (uint32_t)(yt >> 32), t2 = (uint32_t)(lt >> 32),
+                           t3 = (uint32_t)(pt >> 32), t4 = (uint32_t)(best >> 32);
+            tags = t0 == jid && t1 == jid && t2 == jid && t3 == jid && t4 >= jid;
+            // a later job's word: the claim's job is over; an older one's: the
+            // descriptor is still on its way (looked at again, a bounded number
+            // of times: the owner scans a chunk that nobody answers)
+            if (!tags && (max(max(t0, t1), max(t2, t3)) > jid || look == 256)) {
                 J->jid = 0;
                 return 0;
             }
         }
         // the pair's strings: the launch's pair table, read once per pair
-        if (J->pq != (int32_t)(uint32_t)pt) {
-            const PairDesc &D = P.pairs[(uint32_t)pt];
+        const uint32_t pi = (uint32_t)pt & PAIR_MASK;
+        if (J->pq != (int32_t)pi) {
+            const PairDesc &D = P.pairs[pi];
             J->A = D.A;
             J->B = D.B;
             J->n = (int32_t)D.n;
             J->m = (int32_t)D.m;
-            J->pq = (int32_t)(uint32_t)pt;
+            J->pq = (int32_t)pi;
         }
+        J->chunk = chunk_bytes((uint32_t)pt >> 31);
         J->x = (int32_t)(uint32_t)xt;
         J->y = (int32_t)(uint32_t)yt;
         J->lim = (int32_t)(uint32_t)lt;
@@ -428,49 +464,61 @@ __device__ __forceinline__ int claim_go(const LvArgs &P, const Smem S, JobSlot *
         if (J->x < 0 || J->y < 0 || J->lim < 0 || (int64_t)J->x + J->lim > J->n || (int64_t)J->y + J->lim > J->m ||
             !J->A || !J->B) {
             J->jid = 0;
-            if (S.err && atomicCAS(S.err, 0u, 7u) == 0u) {
-                S.diag[0] = 7;
-                S.diag[1] = blockIdx.x;
-                S.diag[2] = (unsigned long long)J->x;
-                S.diag[3] = (unsigned long long)J->y;
-                S.diag[4] = (unsigned long long)J->lim;
-                S.diag[5] = (unsigned long long)J->n;
-                S.diag[6] = (unsigned long long)J->m;
+            if (atomicCAS(&P.ctl->error, 0u, 7u) == 0u) {
+                P.ctl->diag[0] = 7;
+                P.ctl->diag[1] = blockIdx.x;
+                P.ctl->diag[2] = (unsigned long long)J->x;
+                P.ctl->diag[3] = (unsigned long long)J->y;
+                P.ctl->diag[4] = (unsigned long long)J->lim;
+                P.ctl->diag[5] = (unsigned long long)J->n;
+                P.ctl->diag[6] = (unsigned long long)J->m;
             }
             return 0;
         }
     } else if (best == ~0ull) {
         best = ld_relaxed_u64(&sl->result);
     }
-    const int64_t cs = c * (int64_t)CHUNK_BYTES;
+    const int64_t cs = c * (int64_t)J->chunk;
     return cs < result_of(best, jid, J->lim) ? 1 : 0;
 }
 
 // The first mismatch of A[x0..x0+len) vs B[y0..) (len <= CHUNK_BYTES), or
-// -1: by bulk copies into the CTA's stage when it has one, else by one
-// register sweep.  Whole CTA.  (A stage wait that gave up has set the launch
-// status; the chunk then counts as equal and the launch reports the timeout.)
+// -1: by bulk copies into the CTA's stage when it has one, else (and for small
+// chunks) by register sweeps.  Whole CTA.  (A
+// stage wait that gave up has set the launch status; the chunk then counts as
+// equal and the launch reports the timeout.)
 __device__ __forceinline__ int64_t chunk_scan(const LvArgs &P, const Smem S, const uint8_t *A, int64_t n,
                                               const uint8_t *B, int64_t m, int64_t x0, int64_t y0, int64_t len)
 {
-    if (S.stg) {
-        const int64_t r = stage_scan<CHUNK_BYTES>(stage_of(S.stg), A, n, B, m, x0, y0, len, S.smin, P.spin_ns, S.err);
+    if (len <= 0)
+        return -1;
+    if (len > SMALL_CHUNK && S.stg()) {
+        const int64_t r = stage_scan<CHUNK_BYTES>(stage_of(S.stg()), A, n, B, m, x0, y0, len, S.smin(), P.spin_ns, &P.ctl->error);
         return r >= 0 ? r : -1;
     }
-    return sweep_scan<CHUNK_BYTES / (CTA_THREADS * 16)>(A, n, B, m, x0, y0, len, S.smin);
+    if (len <= SMALL_CHUNK)
+        return sweep_scan<1>(A, n, B, m, x0, y0, len, S.smin());
+    constexpr int U = CHUNK_BYTES / (CTA_THREADS * 16);
+    constexpr int64_t STEP = CTA_THREADS * 16 * U - 16;
+    for (int64_t o = 0; o < len; o += STEP) {
+        const int64_t r = sweep_scan<U>(A, n, B, m, x0 + o, y0 + o, min(STEP, len - o), S.smin());
+        if (r >= 0)
+            return o + r;
+    }
+    return -1;
 }
 
-// The whole CTA scans claimed chunk c of job jid, cached in S.jd (when go),
+// The whole CTA scans claimed chunk c of job jid, cached in S.jd() (when go),
 // and answers the claim.
 __device__ __forceinline__ void scan_claim(const LvArgs &P, const Smem S, JobSlot *sl, uint32_t jid, int64_t c,
                                            int go)
 {
     int64_t r = -1;
     if (go) {
-        const JobDesc J = *S.jd;
-        const int64_t cs = c * (int64_t)CHUNK_BYTES;
+        const JobDesc J = *S.jd();
+        const int64_t cs = c * (int64_t)J.chunk;
         const int64_t q = chunk_scan(P, S, J.A, J.n, J.B, J.m, J.x + cs, J.y + cs,
-                                     min((int64_t)CHUNK_BYTES, (int64_t)J.lim - cs));
+                                     min((int64_t)J.chunk, (int64_t)J.lim - cs));
         r = q >= 0 ? cs + q : -1;
     }
     if (threadIdx.x == 0)
@@ -513,20 +561,20 @@ __device__ int claim_loop(const LvArgs &P, const Smem S, JobSlot *sl, int s, uns
             const bool ready = wake && wake_ready(wake);
             const int valid = claim_valid(w) ? 1 : 0;
             const int go = valid ? claim_go(P, S, sl, s, w, best) : 0;
-            S.bc[0] = valid;
-            S.bc[3] = go;
-            S.bcl[0] = (long long)w;
+            S.bc()[0] = valid;
+            S.bc()[3] = go;
+            S.bcl()[0] = (long long)w;
             // the next claim and a look at the result, both in flight during
             // the scan below (this claim is still unanswered: the job cannot
             // change meanwhile)
             const bool next = go && !ready && made + 1 < budget;
             w = next ? atomicAdd(&sl->claim, 1ull) : 0ull;
             best = next ? ld_relaxed_u64(&sl->result) : ~0ull;
-            S.bc[4] = next;
+            S.bc()[4] = next;
         }
         __syncthreads();
-        const int valid = S.bc[0], go = S.bc[3], more = S.bc[4];
-        const unsigned long long wc = (unsigned long long)S.bcl[0];
+        const int valid = S.bc()[0], go = S.bc()[3], more = S.bc()[4];
+        const unsigned long long wc = (unsigned long long)S.bcl()[0];
         __syncthreads();
         if (!valid)
             break;
@@ -546,7 +594,7 @@ __device__ int claim_loop(const LvArgs &P, const Smem S, JobSlot *sl, int s, uns
 __device__ int claim_loop2(const LvArgs &P, const Smem S, JobSlot *sl, int s, int budget, const Wake *wake)
 {
     const int tid = threadIdx.x;
-    const Stage T0 = stage_of(S.stg), T1 = stage_of(S.stg + STAGE_STRIDE);
+    const Stage T0 = stage_of(S.stg()), T1 = stage_of(S.stg() + STAGE_STRIDE);
     unsigned long long wn = 0, bestn = ~0ull; // thread 0: the claim in flight, the result read with it
     unsigned long long pre[4] = {0, 0, 0, 0};  // thread 0: the descriptor words read with the first claim
     if (tid == 0) {
@@ -569,37 +617,43 @@ __device__ int claim_loop2(const LvArgs &P, const Smem S, JobSlot *sl, int s, in
             const int ng = nv ? claim_go(P, S, sl, s, wn, bestn, made + pvalid == 0 ? pre : nullptr) : 0;
             const unsigned long long wc = wn;
             // 2. its copies, in flight while the pending chunk is compared
-            if (ng) {
-                const JobDesc &J = *S.jd;
-                const int64_t cs = (int64_t)(uint32_t)wc * (int64_t)CHUNK_BYTES;
+            if (ng && S.jd()->chunk > SMALL_CHUNK) {
+                const JobDesc &J = *S.jd();
+                const int64_t cs = (int64_t)(uint32_t)wc * J.chunk;
                 stage_issue(sn ? T1 : T0, J.A, J.n, J.B, J.m, J.x + cs, J.y + cs,
-                            min((int64_t)CHUNK_BYTES, (int64_t)J.lim - cs), true);
+                            min((int64_t)J.chunk, (int64_t)J.lim - cs), true);
             }
             // 3. the claim after it, in flight meanwhile
             const bool ready = wake && wake_ready(wake);
             const bool more = ng && !ready && made + pvalid + nv < budget;
             wn = more ? atomicAdd(&sl->claim, 1ull) : 0ull;
             bestn = more ? ld_relaxed_u64(&sl->result) : ~0ull;
-            S.bc[0] = nv;
-            S.bc[3] = ng;
-            S.bcl[0] = (long long)wc;
+            S.bc()[0] = nv;
+            S.bc()[3] = ng ? (S.jd()->chunk > SMALL_CHUNK ? 1 : 2) : 0;
+            S.bcl()[0] = (long long)wc;
         }
         __syncthreads();
-        const int nv = S.bc[0], ng = S.bc[3];
-        const unsigned long long wcn = (unsigned long long)S.bcl[0];
+        const int nv = S.bc()[0], ng = S.bc()[3]; // (1: staged, 2: a small chunk, swept when its turn comes)
+        const unsigned long long wcn = (unsigned long long)S.bcl()[0];
         const int64_t nc = (int64_t)(uint32_t)wcn;
         __syncthreads();
         // 4. the pending chunk: compared (when worth it) and answered
         if (pvalid) {
             int64_t r = -1;
-            if (pgo) {
-                const JobDesc J = *S.jd;
+            if (pgo == 2) {
+                const JobDesc J = *S.jd();
+                const int64_t cs = pc * (int64_t)J.chunk;
+                const int64_t q = chunk_scan(P, S, J.A, J.n, J.B, J.m, J.x + cs, J.y + cs,
+                                             min((int64_t)SMALL_CHUNK, (int64_t)J.lim - cs));
+                r = q >= 0 ? cs + q : -1;
+            } else if (pgo) {
+                const JobDesc J = *S.jd();
                 const int64_t cs = pc * (int64_t)CHUNK_BYTES;
                 const Stage T = ps ? T1 : T0;
                 const StagedChunk K = stage_issue(T, J.A, J.n, J.B, J.m, J.x + cs, J.y + cs,
                                                   min((int64_t)CHUNK_BYTES, (int64_t)J.lim - cs), false);
-                if (stage_wait(T, P.spin_ns, S.err)) {
-                    const int64_t q = stage_compare(T, K, S.smin);
+                if (stage_wait(T, P.spin_ns, &P.ctl->error)) {
+                    const int64_t q = stage_compare(T, K, S.smin());
                     r = q >= 0 ? cs + q : -1;
                 }
             }
@@ -658,7 +712,7 @@ __device__ __forceinline__ int pick_slot(const LvArgs &P)
 // `budget` claims.  Returns true if a claim was made.
 __device__ __forceinline__ bool serve_slot(const LvArgs &P, const Smem S, int s, int budget, const Wake *wake)
 {
-    if (budget > 1 && S.stg && P.stage >= 2)
+    if (budget > 1 && S.stg() && P.stage >= 2)
         return claim_loop2(P, S, &P.slots[s], s, budget, wake) > 0;
     return claim_loop(P, S, &P.slots[s], s, 0ull, budget, wake) > 0;
 }
@@ -673,28 +727,27 @@ __device__ __forceinline__ bool serve_slot(const LvArgs &P, const Smem S, int s,
 // then takes its bit out of the active mask and returns; claims that come
 // later find their chunk past the result and answer at once.
 __device__ __noinline__ int64_t run_job(const LvArgs &P, const Smem S, const Pair Q, int64_t x, int64_t y,
-                                        int64_t lim)
+                                        int64_t lim, bool small)
 {
     const int tid = threadIdx.x, lane = tid & 31;
-    const uint32_t nch = (uint32_t)((lim + CHUNK_BYTES - 1) / CHUNK_BYTES);
-    const int ring = *S.jring;
+    const uint32_t nch = (uint32_t)((lim + chunk_bytes(small) - 1) / chunk_bytes(small));
+    const int ring = *S.jring();
     const int sidx = (int)blockIdx.x * JOB_RING + ring;
     JobSlot *sl = &P.slots[sidx];
     const int word = sidx >> 6;
     const unsigned long long bit = 1ull << (sidx & 63);
     // ------------------------------------------------ publish
     if (tid == 0) {
-        *S.jring = (ring + 1) % JOB_RING;
-        uint32_t jid = (uint32_t)(ld_relaxed_u64(&sl->claim) >> 32) + 1u;
-        jid = jid ? jid : 1u;
+        *S.jring() = (ring + 1) % JOB_RING;
+        const uint32_t jid = (uint32_t)++S.jids()[ring]; // (this CTA's alone to count)
         const unsigned long long tg = (unsigned long long)jid << 32;
-        sl->xt = tg | (uint32_t)x;
-        sl->yt = tg | (uint32_t)y;
-        sl->lt = tg | (uint32_t)lim;
-        sl->pt = tg | (uint32_t)Q.q;
-        sl->result = tg | (uint32_t)~(uint32_t)lim;
+        st_relaxed_u64(&sl->xt, tg | (uint32_t)x);
+        st_relaxed_u64(&sl->yt, tg | (uint32_t)y);
+        st_relaxed_u64(&sl->lt, tg | (uint32_t)lim);
+        st_relaxed_u64(&sl->pt, tg | (uint32_t)small << 31 | (uint32_t)Q.q);
+        st_relaxed_u64(&sl->result, tg | (uint32_t)~(uint32_t)lim);
         // the CTA's own cache holds the job: no read back
-        JobDesc *J = S.jd;
+        JobDesc *J = S.jd();
         J->A = Q.A;
         J->B = Q.B;
         J->n = (int32_t)Q.n;
@@ -705,15 +758,14 @@ __device__ __noinline__ int64_t run_job(const LvArgs &P, const Smem S, const Pai
         J->lim = (int32_t)lim;
         J->jid = jid;
         J->slot = sidx;
-        // count 1: chunk 0 is the CTA's own claim; the descriptor is visible
-        // before the claim word (release), which opens the job, and before
-        // the active bit (release)
-        st_release_u64(&sl->claim, tg | 1ull);
-        asm volatile("red.release.gpu.global.or.b64 [%0], %1;" ::"l"(&P.ctl->active[word]), "l"(bit) : "memory");
-        S.bcl[2] = (long long)tg;
+        J->chunk = chunk_bytes(small);
+        // count 1: chunk 0 is the CTA's own claim
+        st_relaxed_u64(&sl->claim, tg | 1ull);
+        asm volatile("red.relaxed.gpu.global.or.b64 [%0], %1;" ::"l"(&P.ctl->active[word]), "l"(bit) : "memory");
+        S.bcl()[2] = (long long)tg;
     }
     __syncthreads();
-    const unsigned long long w0 = (unsigned long long)S.bcl[2];
+    const unsigned long long w0 = (unsigned long long)S.bcl()[2];
     const uint32_t jid = (uint32_t)(w0 >> 32);
     __syncthreads();
     claim_loop(P, S, sl, sidx, w0, 1, nullptr, w0 | (uint32_t)~(uint32_t)lim); // chunk 0
@@ -776,15 +828,15 @@ __device__ __noinline__ int64_t run_job(const LvArgs &P, const Smem S, const Pai
                 act = __shfl_sync(0xffffffffu, act, 0);
             }
             if (lane == 0) {
-                S.bc[5] = act;
-                S.bcl[1] = (long long)best;
-                S.bc[6] = (int)base;
+                S.bc()[5] = act;
+                S.bcl()[1] = (long long)best;
+                S.bc()[6] = (int)base;
             }
         }
         __syncthreads();
-        const int act = S.bc[5];
-        const int64_t best = S.bcl[1];
-        const int64_t cb = S.bc[6];
+        const int act = S.bc()[5];
+        const int64_t best = S.bcl()[1];
+        const int64_t cb = S.bc()[6];
         __syncthreads();
         if (act == 2) {
             if (tid == 0)
@@ -811,28 +863,32 @@ __device__ __noinline__ int64_t run_job(const LvArgs &P, const Smem S, const Pai
 // between two calls).
 constexpr int64_t ALONE_BYTES = 64 * 1024;
 constexpr int RUN_BYTES = 32 * 1024;
+constexpr int SMALL_RUN = 256 * 1024;
 __device__ __noinline__ int64_t long_slide(const LvArgs &P, const Smem S, const Pair Q, int64_t x0,
                                            int64_t y0, int64_t lim0)
 {
-    const int mean = *S.run;
+    const int mean = *S.run();
     const int64_t loc = min(lim0, max(mean <= RUN_BYTES ? ALONE_BYTES : (int64_t)0,
                                       (int64_t)max(0, P.local_chunks) * CHUNK_BYTES));
     int64_t r = -1;
     if (loc > 0)
-        r = stream_sweep<2>(Q.A, Q.n, Q.B, Q.m, x0, y0, loc, S.smin);
+        r = stream_sweep<2>(Q.A, Q.n, Q.B, Q.m, x0, y0, loc, S.smin());
     int64_t off = loc;
     while (r < 0 && off < lim0) {
-        const int64_t len = min(lim0 - off, (int64_t)JOB_MAX_CHUNKS * CHUNK_BYTES);
-        const int64_t q = run_job(P, S, Q, x0 + off, y0 + off, len);
+        // slides that run to a few hundred KB go in small chunks, one load a
+        // thread: more CTAs share them, and a chunk takes half as long
+        const bool small = mean <= SMALL_RUN;
+        const int64_t len = min(lim0 - off, (int64_t)JOB_MAX_CHUNKS * chunk_bytes(small));
+        const int64_t q = run_job(P, S, Q, x0 + off, y0 + off, len, small);
         if (q < len)
             r = off + q;
         off += len;
     }
     if (r < 0)
         r = lim0;
-    __syncthreads(); // every thread has read *S.run and the sweep's answer
+    __syncthreads(); // every thread has read *S.run() and the sweep's answer
     if (threadIdx.x == 0)
-        *S.run = mean + (((int)min(r, (int64_t)1 << 24) - mean) >> 2);
+        *S.run() = mean + (((int)min(r, (int64_t)1 << 24) - mean) >> 2);
     return r;
 }
 
@@ -872,10 +928,10 @@ __device__ int group_barrier(const LvArgs &P, GroupCtl *gc, uint32_t *count, uin
                 }
             }
         }
-        S.bc[2] = ok;
+        S.bc()[2] = ok;
     }
     __syncthreads();
-    const int ok = S.bc[2];
+    const int ok = S.bc()[2];
     __syncthreads();
     return ok;
 }
@@ -885,59 +941,18 @@ __device__ bool group_sync(const LvArgs &P, GroupCtl *gc, int G, const Smem S)
     return group_barrier(P, gc, &gc->bar_count, &gc->bar_gen, G, false, S) == 1;
 }
 
-constexpr int OCAP = 1024;     // open slides listed per round (pipelined rounds)
-constexpr int DCAP = 3 * OCAP; // deferred diagonals: neighbours of open ones
-
 size_t lv_tiles_smem_bytes(int smax, int h, int stage)
 {
     (void)h;
-    // two frontier buffers and the open-slide list, each smax + 2*HMAX + 2;
-    // two open lists of OCAP (diagonal, start row); DCAP deferred diagonals;
-    // then, with a stage, one chunk's bulk-copy staging (128-byte aligned)
-    return 256 + 3 * sizeof(int32_t) * ((size_t)smax + 2 * HMAX + 2) +
-           sizeof(int32_t) * (4 * (size_t)OCAP + DCAP) + (stage ? 128 + (size_t)stage * STAGE_STRIDE : 0);
+    // the header, two frontier buffers of smax + 2*HMAX + 2, two open lists of
+    // OCAP (diagonal, start row), DCAP deferred diagonals; then the stages
+    // (128-byte aligned)
+    return HEADER + 2 * sizeof(int32_t) * ((size_t)smax + 2 * HMAX + 2) + sizeof(int32_t) * (4 * (size_t)OCAP + DCAP) +
+           (stage ? 128 + (size_t)stage * STAGE_STRIDE : 0);
 }
 
 // The frontier of round r (buffers alternate by parity).
-__device__ __forceinline__ int32_t *frontier(const Smem S, int64_t r) { return (r & 1) ? S.F1 : S.F0; }
-
-__device__ Smem carve(const LvArgs &P)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Smem S;
-    unsigned char *p = smem_raw;
-    S.smin = reinterpret_cast<unsigned long long *>(p);
-    S.bcl = reinterpret_cast<long long *>(p + 16);
-    S.n1 = reinterpret_cast<int *>(p + 64);
-    S.bc = S.n1 + 4;
-    S.nL = reinterpret_cast<int *>(p + 128);
-    S.nD = S.nL + 2;
-    S.left = S.nL + 4;
-    S.kf = S.nL + 6;
-    S.nR = S.nL + 7;
-    S.jd = reinterpret_cast<JobDesc *>(p + 192);
-    S.jring = reinterpret_cast<int *>(p + 48);
-    S.run = reinterpret_cast<int *>(p + 72);
-    // p + 176: lone (lean_slides); p + 184: the tile's lead at an epoch change
-    p += 256;
-    S.lcap = P.smax + 2 * HMAX + 2;
-    S.ld = reinterpret_cast<int32_t *>(p);
-    p += sizeof(int32_t) * S.lcap;
-    S.F0 = reinterpret_cast<int32_t *>(p);
-    p += sizeof(int32_t) * (P.smax + 2 * HMAX + 2);
-    S.F1 = reinterpret_cast<int32_t *>(p);
-    p += sizeof(int32_t) * (P.smax + 2 * HMAX + 2);
-    S.Ld0 = reinterpret_cast<int32_t *>(p);
-    S.Ld1 = S.Ld0 + OCAP;
-    S.Lc0 = S.Ld1 + OCAP;
-    S.Lc1 = S.Lc0 + OCAP;
-    S.D = S.Lc1 + OCAP;
-    p = reinterpret_cast<unsigned char *>(S.D + DCAP);
-    S.stg = P.stage ? reinterpret_cast<unsigned char *>(((uintptr_t)p + 127) & ~(uintptr_t)127) : nullptr;
-    S.err = &P.ctl->error;
-    S.diag = P.ctl->diag;
-    return S;
-}
+__device__ __forceinline__ int32_t *frontier(const Smem S, int64_t r) { return (r & 1) ? S.F1() : S.F0(); }
 
 struct Tile {
     int64_t lo_all, hi_all, S;
@@ -1090,10 +1105,10 @@ __device__ __forceinline__ void cta_slides(const LvArgs &P, const Smem S, const 
         if (tid < 32) {
             const int64_t l = open_limit(P, Q, c, d, C, false);
             if (tid == 0)
-                S.bcl[3] = l;
+                S.bcl()[3] = l;
         }
         __syncthreads();
-        const int64_t lim = S.bcl[3];
+        const int64_t lim = S.bcl()[3];
         __syncthreads();
         const int64_t rr = long_slide(P, S, Q, c, c + d, lim - c);
         C.longs++;
@@ -1108,7 +1123,8 @@ __device__ __forceinline__ void cta_slides(const LvArgs &P, const Smem S, const 
 
 // What one block of rounds adds to the counters, and whether it found k.
 struct BlockOut {
-    unsigned long long slide, mism, hashq, coll, longs, opens, tm_round, tm_open;
+    unsigned long long slide, mism;
+    uint32_t hashq, coll, longs, opens;
     int fin;
 };
 
@@ -1131,12 +1147,12 @@ __device__ __forceinline__ RoundArgs round_args(const LvArgs &P, const Smem S, c
     RA.b = b;
     RA.err = &P.ctl->error;
     RA.diag = P.ctl->diag;
-    RA.n1 = S.nL + (tau & 1);
-    RA.open = (tau & 1) ? S.Ld1 : S.Ld0;
-    RA.open_c = (tau & 1) ? S.Lc1 : S.Lc0;
+    RA.n1 = S.nL() + (tau & 1);
+    RA.open = (tau & 1) ? S.Ld1() : S.Ld0();
+    RA.open_c = (tau & 1) ? S.Lc1() : S.Lc0();
     RA.ocap = OCAP;
-    RA.defer = S.D;
-    RA.nd = S.nD + (tau & 1);
+    RA.defer = S.D();
+    RA.nd = S.nD() + (tau & 1);
     RA.list = nullptr;
     RA.nlist = 0;
     RA.tid = threadIdx.x;
@@ -1185,10 +1201,10 @@ __device__ __forceinline__ BlockOut run_block(const LvArgs &P, const Smem S, con
         }
     };
     if (tid == 0) {
-        S.nL[0] = S.nL[1] = 0;
-        S.nD[0] = S.nD[1] = 0;
-        S.left[0] = S.left[1] = 0;
-        S.nR[0] = S.nR[1] = 0;
+        S.nL()[0] = S.nL()[1] = 0;
+        S.nD()[0] = S.nD()[1] = 0;
+        S.left()[0] = S.left()[1] = 0;
+        S.nR()[0] = S.nR()[1] = 0;
     }
     __syncthreads();
     int r = 0;
@@ -1205,14 +1221,14 @@ __device__ __forceinline__ BlockOut run_block(const LvArgs &P, const Smem S, con
         for (int64_t d = max(ra, bhi + 1) + tid; d < rb; d += nt)
             cur[d - off] = NEG;
         const int pp = (int)((tau - 1) & 1);
-        int32_t *Ldp = pp ? S.Ld1 : S.Ld0;
-        const int32_t *Lcp = pp ? S.Lc1 : S.Lc0;
-        const int nlp = r > 0 ? min(S.nL[pp], OCAP) : 0;
+        int32_t *Ldp = pp ? S.Ld1() : S.Ld0();
+        const int32_t *Lcp = pp ? S.Lc1() : S.Lc0();
+        const int nlp = r > 0 ? min(S.nL()[pp], OCAP) : 0;
         // -------- phase 1: the slides of round tau - 1 || round tau
         if (slider) {
             const RoundArgs RN = round_args(P, S, Q, tau, max(ra, blo), min(rb - 1, bhi), off, a, b);
-            warp_slides(P, Q, prev, off, Ldp, Lcp, nlp, a, b, sli, nsl, C, S.left + (tau & 1), &RN,
-                        S.nR + (tau & 1));
+            warp_slides(P, Q, prev, off, Ldp, Lcp, nlp, a, b, sli, nsl, C, S.left() + (tau & 1), &RN,
+                        S.nR() + (tau & 1));
         } else {
             RoundArgs RA = round_args(P, S, Q, tau, max(ra, blo), min(rb - 1, bhi), off, a, b);
             RA.tid = tid - 32 * sli;
@@ -1226,26 +1242,26 @@ __device__ __forceinline__ BlockOut run_block(const LvArgs &P, const Smem S, con
         }
         __syncthreads();
         // -------- phase 2: slides the warp left open, then the deferred diagonals
-        if (nlp > 0 && S.left[tau & 1])
+        if (nlp > 0 && S.left()[tau & 1])
             cta_slides(P, S, Q, prev, off, Ldp, Lcp, nlp, a, b, C);
-        const int nd = S.nD[tau & 1];                   // deferred diagonals listed
-        const bool marked = nd > S.nR[tau & 1];          // not all computed by a slider warp
+        const int nd = S.nD()[tau & 1];                   // deferred diagonals listed
+        const bool marked = nd > S.nR()[tau & 1];          // not all computed by a slider warp
         if (tid == 0) {
             // round tau - 1's list is consumed (every thread read its count
             // before the first barrier); the same parity's counts serve round
             // tau + 1 (round tau - 1's deferred count was last read before
             // the second barrier of round tau - 1)
-            S.nL[pp] = 0;
-            S.nD[pp] = 0;
-            S.left[pp] = 0;
-            S.nR[pp] = 0;
+            S.nL()[pp] = 0;
+            S.nD()[pp] = 0;
+            S.left()[pp] = 0;
+            S.nR()[pp] = 0;
             // round tau - 1 is final here for thread 0: the slider's rows
             // before the first barrier, the CTA's slides by thread 0 itself
-            *S.kf = r > 0 && hit(tau - 1);
+            *S.kf() = r > 0 && hit(tau - 1);
         }
         if (marked) {
             RoundArgs RA = round_args(P, S, Q, tau, 0, -1, off, a, b);
-            RA.list = S.D;
+            RA.list = S.D();
             RA.nlist = nd;
             const RoundCount rc = tile_round<1, true, true>(RA);
             C.slide += rc.slide;
@@ -1254,7 +1270,7 @@ __device__ __forceinline__ BlockOut run_block(const LvArgs &P, const Smem S, con
         __syncthreads();
         // round tau - 1 is final now (round tau is tested in the next round,
         // or below if tau ends the block)
-        if (*S.kf)
+        if (*S.kf())
             kfound = tau - 1;
         if (dump) {
             // round tau + 1 overwrites this buffer
@@ -1262,16 +1278,17 @@ __device__ __forceinline__ BlockOut run_block(const LvArgs &P, const Smem S, con
                 dump_row(tau - 1);
             __syncthreads();
         }
-        C.tm[0] += clock64() - tr0;
+        if (tid == 0)
+            S.tm()[0] += clock64() - tr0;
     }
     // -------- the last computed round's open slides: all warps
     const uint64_t to0 = clock64();
     const int64_t tl = t + r - 1;
     if (kfound < 0 || kfound == tl) {
         const int pl = (int)(tl & 1);
-        int32_t *Ldl = pl ? S.Ld1 : S.Ld0;
-        const int32_t *Lcl = pl ? S.Lc1 : S.Lc0;
-        const int nll = min(S.nL[pl], OCAP);
+        int32_t *Ldl = pl ? S.Ld1() : S.Ld0();
+        const int32_t *Lcl = pl ? S.Lc1() : S.Lc0();
+        const int nll = min(S.nL()[pl], OCAP);
         if (nll > 0) {
             warp_slides(P, Q, frontier(S, tl), off, Ldl, Lcl, nll, a, b, warp, nw, C, nullptr);
             __syncthreads();
@@ -1282,13 +1299,14 @@ __device__ __forceinline__ BlockOut run_block(const LvArgs &P, const Smem S, con
         if (kfound < 0 && hit(tl))
             kfound = tl;
     }
-    C.tm[1] += clock64() - to0;
+    if (tid == 0)
+        S.tm()[1] += clock64() - to0;
     if (kfound >= 0 && tid == 0) {
         atomicMin(&gc->done_k, (unsigned long long)kfound);
         res[R_K] = (unsigned long long)kfound;
     }
     __syncthreads();
-    return BlockOut{C.slide, C.mism, C.hashq, C.coll, C.longs, C.opens, C.tm[0], C.tm[1], kfound >= 0 ? 1 : 0};
+    return BlockOut{C.slide, C.mism, C.hashq, C.coll, C.longs, C.opens, kfound >= 0 ? 1 : 0};
 }
 
 // A lone slide this long is worth the whole CTA (one step of stream_sweep).
@@ -1307,7 +1325,7 @@ __device__ __forceinline__ void lean_slides(const LvArgs &P, const Smem S, const
     // the next lone one then goes to the whole CTA at once (its job opens
     // without the warp's step first): on the alignment path, slides long
     // and short come in runs
-    int *lone = reinterpret_cast<int *>(reinterpret_cast<unsigned char *>(S.jring) + 128);
+    int *lone = S.lone();
     const bool direct = nlo == 1 && *lone != 0;
     if (direct && !Q.hash) {
         const int64_t d = Ld[0], c = Lc[0], lim = min(Q.n - c, Q.m - c - d);
@@ -1327,15 +1345,15 @@ __device__ __forceinline__ void lean_slides(const LvArgs &P, const Smem S, const
         cta_slides(P, S, Q, cur, off, Ld, Lc, nlo, a, b, C);
     } else {
         const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        warp_slides(P, Q, cur, off, Ld, Lc, nlo, a, b, warp, nw, C, S.left + pr);
+        warp_slides(P, Q, cur, off, Ld, Lc, nlo, a, b, warp, nw, C, S.left() + pr);
         __syncthreads();
-        if (S.left[pr])
+        if (S.left()[pr])
             cta_slides(P, S, Q, cur, off, Ld, Lc, nlo, a, b, C);
     }
     if (threadIdx.x == 0) {
         if (nlo == 1)
-            *lone = direct ? (cur[Ld[0] - off] - Lc[0] > LONE_BYTES) : S.left[pr];
-        S.left[pr] = 0;
+            *lone = direct ? (cur[Ld[0] - off] - Lc[0] > LONE_BYTES) : S.left()[pr];
+        S.left()[pr] = 0;
     }
     __syncthreads();
 }
@@ -1358,8 +1376,8 @@ __device__ __forceinline__ BlockOut run_block_lean(const LvArgs &P, const Smem S
     Counters C;
     int64_t kfound = -1;
     if (tid == 0) {
-        S.nL[0] = S.nL[1] = 0;
-        S.left[0] = S.left[1] = 0;
+        S.nL()[0] = S.nL()[1] = 0;
+        S.left()[0] = S.left()[1] = 0;
     }
     __syncthreads();
     int r = 0;
@@ -1371,9 +1389,9 @@ __device__ __forceinline__ BlockOut run_block_lean(const LvArgs &P, const Smem S
         const int32_t blo = (int32_t)max(-tau, -n), bhi = (int32_t)min(tau, m);
         int32_t *cur = frontier(S, tau);
         const int32_t *prev = frontier(S, tau - 1);
-        int32_t *Ld = pr ? S.Ld1 : S.Ld0;
-        int32_t *Lc = pr ? S.Lc1 : S.Lc0;
-        int *nl = S.nL + pr;
+        int32_t *Ld = pr ? S.Ld1() : S.Ld0();
+        int32_t *Lc = pr ? S.Lc1() : S.Lc0();
+        int *nl = S.nL() + pr;
         for (int32_t d = ra + tid; d < rb; d += (int32_t)blockDim.x) {
             if (d < blo || d > bhi) {
                 cur[d - off] = NEG;
@@ -1384,7 +1402,7 @@ __device__ __forceinline__ BlockOut run_block_lean(const LvArgs &P, const Smem S
                     cc = min(max(x1, max(x2, x3) + 1), d <= mn ? n32 : m32 - d);
                 }
                 if (cc < 0 || cc + d < 0) {
-                    record_bad_row(S.err, S.diag, tau, prev, (int32_t)off, d, cc);
+                    record_bad_row(&P.ctl->error, P.ctl->diag, tau, prev, (int32_t)off, d, cc);
                     cur[d - off] = NEG;
                 } else {
                     const int32_t full = min(n32 - cc, m32 - cc - d);
@@ -1428,7 +1446,7 @@ __device__ __forceinline__ BlockOut run_block_lean(const LvArgs &P, const Smem S
             }
         }
         if (tid == 0)
-            S.nL[pr ^ 1] = 0; // the other parity's list is free again
+            S.nL()[pr ^ 1] = 0; // the other parity's list is free again
         __syncthreads();
         const int nlo = *nl;
         if (nlo > 0)
@@ -1441,14 +1459,15 @@ __device__ __forceinline__ BlockOut run_block_lean(const LvArgs &P, const Smem S
             for (int64_t e = max(a, -TT) + tid; e < min(b, TT + 1); e += blockDim.x)
                 dump[tau * (2 * TT + 1) + e + TT] = cur[e - off];
         }
-        C.tm[0] += clock64() - tr0;
+        if (tid == 0)
+            S.tm()[0] += clock64() - tr0;
     }
     if (kfound >= 0 && tid == 0) {
         atomicMin(&gc->done_k, (unsigned long long)kfound);
         res[R_K] = (unsigned long long)kfound;
     }
     __syncthreads();
-    return BlockOut{C.slide, C.mism, C.hashq, C.coll, C.longs, C.opens, C.tm[0], C.tm[1], kfound >= 0 ? 1 : 0};
+    return BlockOut{C.slide, C.mism, C.hashq, C.coll, C.longs, C.opens, kfound >= 0 ? 1 : 0};
 }
 
 // Whether a CTA that is about to compute round t leaves the pair.  Once k
@@ -1535,14 +1554,14 @@ __device__ __forceinline__ bool run_pair(const LvArgs &P, const Smem S, const Pa
         return true;
     }
     for (int i = tid; i < P.smax + 2 * HMAX + 2; i += nt) {
-        S.F0[i] = NEG;
-        S.F1[i] = NEG;
+        S.F0()[i] = NEG;
+        S.F1()[i] = NEG;
     }
     if (tid == 0) {
-        *S.n1 = 0;
+        *S.n1() = 0;
         // (nothing known yet: the first slide of a string of 8 MB and more is
         // opened to other CTAs at once)
-        *S.run = (int)(min(n, m) >> 8);
+        *S.run() = (int)(min(n, m) >> 8);
     }
     __syncthreads();
     if (t > 0 && T.has) {
@@ -1562,10 +1581,10 @@ __device__ __forceinline__ bool run_pair(const LvArgs &P, const Smem S, const Pa
                 st = 1;
             else if (ld_acquire(&P.ctl->error) != 0)
                 st = 2;
-            S.bc[1] = st;
+            S.bc()[1] = st;
         }
         __syncthreads();
-        const int stop = S.bc[1];
+        const int stop = S.bc()[1];
         __syncthreads();
         if (stop == 1)
             return true;
@@ -1605,14 +1624,14 @@ __device__ __forceinline__ bool run_pair(const LvArgs &P, const Smem S, const Pa
                             st = 2;
                         }
                     }
-                    S.bc[1] = st;
-                    S.bc[2] = sl;
+                    S.bc()[1] = st;
+                    S.bc()[2] = sl;
                     if (st == 3)
-                        S.bcl[2] = *(volatile uint32_t *)&gc->epoch_t;
+                        S.bcl()[2] = *(volatile uint32_t *)&gc->epoch_t;
                 }
                 __syncthreads();
-                const int st = S.bc[1], sl = S.bc[2];
-                const int64_t et = S.bcl[2];
+                const int st = S.bc()[1], sl = S.bc()[2];
+                const int64_t et = S.bcl()[2];
                 __syncthreads();
                 if (st == 1)
                     return true;
@@ -1660,8 +1679,7 @@ __device__ __forceinline__ bool run_pair(const LvArgs &P, const Smem S, const Pa
                 }
             }
             int32_t *buf = gfb + ((epoch + 1) & 1) * gstride;
-            unsigned long long *lead_s = reinterpret_cast<unsigned long long *>(
-                reinterpret_cast<unsigned char *>(S.jring) + 136);
+            unsigned long long *lead_s = S.lead();
             if (tid == 0)
                 *lead_s = 0ull;
             __syncthreads();
@@ -1731,7 +1749,8 @@ __device__ __forceinline__ bool run_pair(const LvArgs &P, const Smem S, const Pa
                     dst[d - (T.a - h) + 1] = (d >= plo && d <= phi) ? ld_cg(buf + d + kc + 2) : NEG;
             }
             __syncthreads();
-            C.tm[3] += clock64() - te0;
+            if (tid == 0)
+                S.tm()[3] += clock64() - te0;
             if (!T.has)
                 continue;
         }
@@ -1774,8 +1793,6 @@ __device__ __forceinline__ bool run_pair(const LvArgs &P, const Smem S, const Pa
             C.coll += bo.coll;
             C.longs += bo.longs;
             C.opens += bo.opens;
-            C.tm[0] += bo.tm_round;
-            C.tm[1] += bo.tm_open;
             const bool fin = bo.fin != 0;
             if (fin)
                 return true;
@@ -1850,12 +1867,12 @@ __device__ __forceinline__ bool run_pair(const LvArgs &P, const Smem S, const Pa
                     }
                 }
                 if (tid == 0) {
-                    S.bc[1] = st;
-                    S.bc[2] = js;
+                    S.bc()[1] = st;
+                    S.bc()[2] = js;
                 }
             }
             __syncthreads();
-            const int st = S.bc[1], js = S.bc[2];
+            const int st = S.bc()[1], js = S.bc()[2];
             __syncthreads();
             if (st == 1)
                 return true;
@@ -1870,11 +1887,12 @@ __device__ __forceinline__ bool run_pair(const LvArgs &P, const Smem S, const Pa
                 serve_slot(P, S, js, 2, &wk);
             }
         }
-        C.tm[2] += clock64() - tw0;
+        if (tid == 0)
+            S.tm()[2] += clock64() - tw0;
     }
 }
 
-__device__ __forceinline__ void flush_counters(const PairDesc &D, Counters &C, bool first_cta)
+__device__ __forceinline__ void flush_counters(const Smem S, const PairDesc &D, Counters &C, bool first_cta)
 {
     unsigned long long v[7] = {C.slide, C.mism, C.hashq, C.coll, C.longs, C.blocks, C.opens};
     for (int o = 16; o; o >>= 1)
@@ -1890,14 +1908,16 @@ __device__ __forceinline__ void flush_counters(const PairDesc &D, Counters &C, b
     if (threadIdx.x == 0) {
         // counted once per CTA (the values are the CTA's, not per thread)
         if (C.longs)
-            atomicAdd(&D.res[R_LONG], C.longs);
+            atomicAdd(&D.res[R_LONG], (unsigned long long)C.longs);
         if (first_cta)
             D.res[R_WIDE] = C.blocks;
         // phase cycles: the largest over the group's CTAs, and the sum of
         // round + slide cycles (for the average busy time)
         for (int i = 0; i < 4; i++)
-            atomicMax(&D.res[R_T0 + i], C.tm[i]);
-        atomicAdd(&D.res[R_T0 + 4], C.tm[0] + C.tm[1]);
+            atomicMax(&D.res[R_T0 + i], S.tm()[i]);
+        atomicAdd(&D.res[R_T0 + 4], S.tm()[0] + S.tm()[1]);
+        for (int i = 0; i < 4; i++)
+            S.tm()[i] = 0;
         atomicAdd(&D.res[R_T0 + 5], 1ull);
     }
     C = Counters();
@@ -1905,19 +1925,23 @@ __device__ __forceinline__ void flush_counters(const PairDesc &D, Counters &C, b
 
 __global__ void __launch_bounds__(CTA_THREADS, 1) lv_tiles_kernel(LvArgs P)
 {
-    const Smem S = carve(P);
+    const Smem S{P.smax, P.stage};
     if (threadIdx.x == 0) { // no job cached (read before the first group barrier)
-        S.jd->jid = 0;
-        S.jd->slot = -1;
-        S.jd->pq = -1;
-        *S.jring = 0;
-        *reinterpret_cast<int *>(reinterpret_cast<unsigned char *>(S.jring) + 128) = 0;
-        for (int i = 0; S.stg && i < P.stage; i++) {
-            const Stage T = stage_of(S.stg + i * STAGE_STRIDE);
+        S.jd()->jid = 0;
+        S.jd()->slot = -1;
+        S.jd()->pq = -1;
+        *S.jring() = 0;
+        for (int i = 0; i < JOB_RING; i++)
+            S.jids()[i] = 0;
+        for (int i = 0; i < 4; i++)
+            S.tm()[i] = 0;
+        *S.lone() = 0;
+        for (int i = 0; S.stg() && i < P.stage; i++) {
+            const Stage T = stage_of(S.stg() + i * STAGE_STRIDE);
             mbar_init(T.bar, 1);
             *T.phase = 0;
         }
-        if (S.stg)
+        if (S.stg())
             fence_mbar_init();
     }
     const uint64_t deadline = gtimer() + P.budget_ns;
@@ -1964,7 +1988,7 @@ __global__ void __launch_bounds__(CTA_THREADS, 1) lv_tiles_kernel(LvArgs P)
             break;
         const PairDesc D = P.pairs[q];
         const bool ok = run_pair(P, S, D, q, gc, gi, G, c0, gfb, kc, deadline, C);
-        flush_counters(D, C, gi == 0);
+        flush_counters(S, D, C, gi == 0);
         if (!ok)
             break;
         if (!group_sync(P, gc, G, S))
@@ -2033,32 +2057,23 @@ __global__ void lcp_query_kernel(const uint8_t *A, int64_t n, const uint8_t *B, 
 // Method 2: every CTA claims chunks of the queries' slots (published by the
 // host: claim = 1 << 32, result = lim) until each slot is exhausted; the
 // answers stay in the slots.
-__device__ uint32_t g_lcp_grid_err; // status word of the test launches below
+__device__ LaunchCtl g_lcp_grid_ctl; // status words of the test launches below
+constexpr int GRID_SMAX = -(2 * HMAX + 2); // (no frontier buffers)
 
 __global__ void __launch_bounds__(CTA_THREADS) lcp_grid_kernel(JobSlot *slots, int nslots, int stage,
                                                                 const PairDesc *pairs)
 {
-    extern __shared__ __align__(128) unsigned char gsm[];
-    __shared__ unsigned long long s_min;
-    __shared__ long long s_bcl[4];
-    __shared__ int s_bc[8];
-    __shared__ JobDesc s_jd;
-    Smem S{};
-    S.smin = &s_min;
-    S.bc = s_bc;
-    S.bcl = s_bcl;
-    S.jd = &s_jd;
-    S.err = &g_lcp_grid_err;
-    S.stg = stage ? gsm : nullptr;
+    const Smem S{GRID_SMAX, stage};
     LvArgs P{};
     P.spin_ns = 2000000000ull;
     P.pairs = pairs;
+    P.ctl = &g_lcp_grid_ctl;
     if (threadIdx.x == 0) {
-        s_jd.jid = 0;
-        s_jd.slot = -1;
-        s_jd.pq = -1;
+        S.jd()->jid = 0;
+        S.jd()->slot = -1;
+        S.jd()->pq = -1;
         if (stage) {
-            const Stage T = stage_of(gsm);
+            const Stage T = stage_of(S.stg());
             mbar_init(T.bar, 1);
             *T.phase = 0;
             fence_mbar_init();
@@ -2082,7 +2097,7 @@ cudaError_t launch_lcp_queries(const uint8_t *A, int64_t n, const uint8_t *B, in
     if (method == 2 || method == 7) {
         // 2: register sweeps; 7: the same claims scanned through a bulk-copy stage
         const int stage = method == 7;
-        const size_t smem = stage ? stage_bytes<CHUNK_BYTES>() : 0;
+        const size_t smem = lv_tiles_smem_bytes(GRID_SMAX, 0, stage);
         if (stage) {
             const cudaError_t e =
                 cudaFuncSetAttribute(lcp_grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -231,3 +231,42 @@ def test_prefix_hash_across_tiles(ctx, orc, length, stride):
         T = ed.ed_prefix_hash_blocked_dev(ctx.h, d, stride)
         want = orc.prefix_hash_blocked(X, stride, base)
     assert np.array_equal(T.cpu().numpy().view(np.uint64), want)
+
+
+@pytest.mark.parametrize("method", [2, 7])
+@pytest.mark.parametrize("sa,sy", [(0, 0), (1, 0), (15, 3), (8, 13), (0, 15)])
+def test_grid_lcp_at_chunk_ends(ctx, orc, method, sa, sy):
+    """The only mismatch in the last bytes of a 16 KiB chunk, at its end and
+    just past it, from start rows at every alignment of A and B."""
+    from paper_2306_17461_gb300 import binding as ed
+
+    n = 3 * 16384 + 100
+    rng = np.random.default_rng(410 + sa)
+    A = rng.integers(0, 4, n, dtype=np.uint8)
+    dA = dev(np.concatenate([np.zeros(sa, np.uint8), A]))[sa:]
+    for off in [16384 - 16, 16384 - 2, 16384 - 1, 16384, 2 * 16384 - 1, 2 * 16384 + 15, n - 1]:
+        B = A.copy()
+        B[off] ^= 1
+        dB = dev(np.concatenate([np.zeros(sy, np.uint8), B]))[sy:]
+        got = ed.ed_lcp_dev(ctx.h, dA, dB, np.array([0]), np.array([0]), method)
+        assert got[0] == off, (method, sa, sy, off)
+
+
+@pytest.mark.parametrize("gap", [3000, 4080, 16 * 1024, 65_535, 65_537, 300_000, 1_100_000])
+def test_slide_lengths_across_the_paths(orc, gap):
+    """Slides around the lengths at which they change hands: a warp, the CTA
+    alone, jobs of small and of large chunks; runs of one length, so that
+    each path's running mean takes hold, then one of another."""
+    from paper_2306_17461_gb300 import binding as ed
+    from paper_2306_17461_gb300 import workloads as W
+
+    rng = np.random.default_rng(gap)
+    reps = max(4, min(40, 3_000_000 // gap))
+    pos = np.cumsum(np.concatenate([np.full(reps, gap), [7, 250_000, 9, 40_000]])) + rng.integers(0, 3, reps + 4)
+    sym = W.Symbols(4)
+    A = sym.draw(rng, int(pos[-1]) + 50_000)
+    B = W.plant(rng, A, pos, sym)
+    want = orc.lv(A, B)
+    for cfg in ({}, {"grid_ctas": 2}, {"help_div": 2, "block_rounds": 16}):
+        with ed.Context(device=0, **cfg) as c:
+            assert c.distance_dev(dev(A), dev(B)) == want, cfg
