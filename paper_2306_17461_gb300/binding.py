@@ -152,6 +152,42 @@ def _host_buf(x):
     return (a.ctypes.data if a.size else None), a.size, a
 
 
+_U8 = np.dtype(np.uint8)
+
+
+def _host_bufs(xs: Sequence):
+    """(pointers, lengths, keepalives) of host byte buffers: _host_buf for
+    each, with numpy byte arrays (the common case) read directly -- the
+    per-buffer Python was most of a batch of short strings."""
+    ptrs, lens, keep = np.zeros(len(xs), np.uint64), np.zeros(len(xs), np.uint64), []
+    for i, x in enumerate(xs):
+        if type(x) is np.ndarray and x.dtype is _U8 and x.flags.c_contiguous:
+            size = x.size
+            if size:
+                ptrs[i] = x.__array_interface__["data"][0]
+                lens[i] = size
+            continue
+        p, size, k = _host_buf(x)
+        ptrs[i], lens[i] = p or 0, size
+        keep.append(k)
+    return ptrs, lens, keep
+
+
+def _dev_bufs(ts: Sequence):
+    """(pointers, lengths) of CUDA byte tensors, each checked as by _dev_buf."""
+    import torch
+
+    T, u8 = torch.Tensor, torch.uint8
+    ptrs, lens = [], []
+    for t in ts:
+        if not isinstance(t, T) or not t.is_cuda or t.dtype != u8 or not t.is_contiguous():
+            _dev_buf(t)  # raises
+        size = t.numel()
+        lens.append(size)
+        ptrs.append(t.data_ptr() if size else 0)
+    return np.array(ptrs, dtype=np.uint64), np.array(lens, dtype=np.uint64)
+
+
 def _dev_buf(t):
     import torch
 
@@ -228,37 +264,24 @@ def ed_last_stats(ctx) -> dict:
     return d
 
 
-def _ptr_array(ptrs):
-    arr = (ctypes.c_void_p * max(1, len(ptrs)))()
-    for i, p in enumerate(ptrs):
-        arr[i] = p
-    return arr
-
-
 def ed_distance_batch_dev(ctx, As: Sequence, Bs: Sequence, stream=None) -> np.ndarray:
     npairs = len(As)
-    pa = [_dev_buf(a) for a in As]
-    pb = [_dev_buf(b) for b in Bs]
-    n = np.array([x[1] for x in pa], dtype=np.uint64)
-    m = np.array([x[1] for x in pb], dtype=np.uint64)
+    pa, n = _dev_bufs(As)
+    pb, m = _dev_bufs(Bs)
     out = np.zeros(max(1, npairs), dtype=np.uint64)
     _check(ctx, load().ed_distance_batch_dev(
-        ctx, npairs, _ptr_array([x[0] for x in pa]), n.ctypes.data if npairs else None,
-        _ptr_array([x[0] for x in pb]), m.ctypes.data if npairs else None,
+        ctx, npairs, *(x.ctypes.data if npairs else None for x in (pa, n, pb, m)),
         out.ctypes.data, _stream_ptr(stream)), "ed_distance_batch_dev")
     return out[:npairs].astype(np.int64)
 
 
 def ed_distance_batch(ctx, As: Sequence, Bs: Sequence) -> np.ndarray:
     npairs = len(As)
-    ha = [_host_buf(a) for a in As]
-    hb = [_host_buf(b) for b in Bs]
-    n = np.array([x[1] for x in ha], dtype=np.uint64)
-    m = np.array([x[1] for x in hb], dtype=np.uint64)
+    pa, n, ka = _host_bufs(As)
+    pb, m, kb = _host_bufs(Bs)
     out = np.zeros(max(1, npairs), dtype=np.uint64)
     _check(ctx, load().ed_distance_batch(
-        ctx, npairs, _ptr_array([x[0] for x in ha]), n.ctypes.data if npairs else None,
-        _ptr_array([x[0] for x in hb]), m.ctypes.data if npairs else None, out.ctypes.data),
+        ctx, npairs, *(x.ctypes.data if npairs else None for x in (pa, n, pb, m)), out.ctypes.data),
         "ed_distance_batch")
     return out[:npairs].astype(np.int64)
 

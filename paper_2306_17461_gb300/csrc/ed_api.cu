@@ -256,6 +256,11 @@ struct ed_ctx {
         border, bnext, bfront, keep, wtiles;
     unsigned long long *h_res = nullptr; // pinned result block
     size_t h_res_cap = 0;
+    // pinned staging of short host strings (HostPacker): two halves, each busy
+    // until its event
+    char *h_stage = nullptr;
+    bool h_stage_failed = false, stage_busy[2] = {false, false};
+    cudaEvent_t stage_ev[2] = {nullptr, nullptr};
     uint64_t hash_base = 0;
     uint64_t pow2[62]{};
     ed_stats last{};
@@ -877,6 +882,11 @@ int ed_destroy(ed_ctx *ctx)
         release(ctx, *b);
     if (ctx->h_res)
         cudaFreeHost(ctx->h_res);
+    if (ctx->h_stage)
+        cudaFreeHost(ctx->h_stage);
+    for (cudaEvent_t e : ctx->stage_ev)
+        if (e)
+            cudaEventDestroy(e);
     if (ctx->ev0)
         cudaEventDestroy(ctx->ev0);
     if (ctx->ev1)
@@ -1393,6 +1403,66 @@ int ed_distance_batch_dev(ed_ctx *ctx, size_t np, const uint8_t *const *A, const
     return batch_core(ctx, np, A, n, B, m, k_out, (cudaStream_t)stream);
 }
 
+// Host strings to consecutive 16-byte aligned places of a device buffer.
+// Short ones gather in the context's pinned staging buffer (two halves in
+// turn) and go in one copy per half: a copy of its own took each of a batch's
+// short strings 2 to 3 us, whatever its length.  Strings of PACK_MAX bytes and
+// more are copied from where they are.
+struct HostPacker {
+    static constexpr size_t HALF = 4u << 20, PACK_MAX = 256u << 10;
+    ed_ctx *ctx;
+    char *dst;
+    size_t at = 0, from = 0; // next place; first byte not copied yet
+    int half = 0;
+    int add(const uint8_t *X, size_t len)
+    {
+        if (!ctx->h_stage && !ctx->h_stage_failed && len < PACK_MAX) {
+            if (cudaMallocHost((void **)&ctx->h_stage, 2 * HALF) != cudaSuccess) {
+                cudaGetLastError(); // (copy each string by itself then)
+                ctx->h_stage = nullptr;
+                ctx->h_stage_failed = true;
+            }
+        }
+        if (len >= PACK_MAX || !ctx->h_stage) {
+            int r = flush();
+            if (r != ED_OK)
+                return r;
+            if (len)
+                CK(cudaMemcpyAsync(dst + at, X, len, cudaMemcpyHostToDevice, ctx->stream));
+            at += (len + 15) & ~(size_t)15;
+            from = at;
+            return ED_OK;
+        }
+        if (at - from + len > HALF) {
+            int r = flush();
+            if (r != ED_OK)
+                return r;
+        }
+        if (at == from && ctx->stage_busy[half]) { // the half's last copy
+            CK(cudaEventSynchronize(ctx->stage_ev[half]));
+            ctx->stage_busy[half] = false;
+        }
+        if (len)
+            std::memcpy(ctx->h_stage + half * HALF + (at - from), X, len);
+        at += (len + 15) & ~(size_t)15;
+        return ED_OK;
+    }
+    int flush()
+    {
+        if (at > from) {
+            CK(cudaMemcpyAsync(dst + from, ctx->h_stage + half * HALF, std::min(at - from, HALF),
+                               cudaMemcpyHostToDevice, ctx->stream));
+            if (!ctx->stage_ev[half])
+                CK(cudaEventCreateWithFlags(&ctx->stage_ev[half], cudaEventDisableTiming));
+            CK(cudaEventRecord(ctx->stage_ev[half], ctx->stream));
+            ctx->stage_busy[half] = true;
+            half ^= 1;
+            from = at;
+        }
+        return ED_OK;
+    }
+};
+
 int ed_distance_batch(ed_ctx *ctx, size_t np, const uint8_t *const *A, const size_t *n,
                       const uint8_t *const *B, const size_t *m, uint64_t *k_out)
 {
@@ -1414,18 +1484,17 @@ int ed_distance_batch(ed_ctx *ctx, size_t np, const uint8_t *const *A, const siz
     if ((r = ensure(ctx, ctx->strA, total + 64)) != ED_OK)
         return r;
     std::vector<const uint8_t *> dA(np), dB(np);
-    size_t off = 0;
+    HostPacker pack{ctx, (char *)ctx->strA.p};
     for (size_t p = 0; p < np; p++) {
-        char *base = (char *)ctx->strA.p;
-        dA[p] = (const uint8_t *)(base + off);
-        if (n[p])
-            CK(cudaMemcpyAsync(base + off, A[p], n[p], cudaMemcpyHostToDevice, ctx->stream));
-        off += (n[p] + 15) & ~(size_t)15;
-        dB[p] = (const uint8_t *)(base + off);
-        if (m[p])
-            CK(cudaMemcpyAsync(base + off, B[p], m[p], cudaMemcpyHostToDevice, ctx->stream));
-        off += (m[p] + 15) & ~(size_t)15;
+        dA[p] = (const uint8_t *)ctx->strA.p + pack.at;
+        if ((r = pack.add(A[p], n[p])) != ED_OK)
+            return r;
+        dB[p] = (const uint8_t *)ctx->strA.p + pack.at;
+        if ((r = pack.add(B[p], m[p])) != ED_OK)
+            return r;
     }
+    if ((r = pack.flush()) != ED_OK)
+        return r;
     return batch_core(ctx, np, dA.data(), n, dB.data(), m, k_out, ctx->stream);
 }
 
