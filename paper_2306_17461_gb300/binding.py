@@ -166,6 +166,7 @@ def _host_bufs(xs: Sequence):
             if size:
                 ptrs[i] = x.__array_interface__["data"][0]
                 lens[i] = size
+            keep.append(x)  # (xs may make its items on the fly)
             continue
         p, size, k = _host_buf(x)
         ptrs[i], lens[i] = p or 0, size

@@ -84,6 +84,30 @@ def test_batch_host_matches_oracle(ctx, orc):
     assert np.array_equal(got, want)
 
 
+@pytest.mark.parametrize("sizes", [
+    [0, 1, 15, 16, 17, 0], [(256 << 10) - 1, 256 << 10, (256 << 10) + 1, 3],  # either side of the staging limit
+    [260_000] * 19 + [300_000, 5] + [262_128] * 17, [65_536] * 130])          # past both staging halves, to their edge
+def test_batch_host_packing(ctx, orc, sizes):
+    """Short host strings gather in a staging buffer, long ones go by
+    themselves; buffers of other kinds, and items made on the fly, are the
+    same strings."""
+    from paper_2306_17461_gb300 import binding as ed
+
+    rng = np.random.default_rng(91)
+    pairs = [W.random_pair(rng, n, min(n // 4, 6), 4) for n in sizes]
+    want = orc.many("lv", pairs)
+    As, Bs = [a for a, _ in pairs], [b for _, b in pairs]
+    assert np.array_equal(ed.ed_distance_batch(ctx.h, As, Bs), want)
+    kinds = [lambda v: v.tobytes(), lambda v: bytearray(v.tobytes()), lambda v: v.astype(np.int64),
+             lambda v: np.repeat(v, 2)[::2], lambda v: v]
+
+    class Lazy(list):
+        def __iter__(self):
+            return (v.copy() for v in list.__iter__(self))
+
+    assert np.array_equal(ed.ed_distance_batch(ctx.h, [kinds[i % 5](a) for i, a in enumerate(As)], Lazy(Bs)), want)
+
+
 def _serve_all(ctx, pairs, timeout_s=120.0):
     from paper_2306_17461_gb300 import binding as ed
 
