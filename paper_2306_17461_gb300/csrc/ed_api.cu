@@ -252,10 +252,12 @@ struct ed_ctx {
     size_t budget = 0;
     size_t held = 0;
     // pool
-    DevBuf strA, strB, gf, ctl, gctl, slots, halo, pdesc, res, dump, hashA, hashB, scan, qx, qy, qo, bpairs,
+    DevBuf strA, strB, gf, ctl, slots, halo, pdesc, dump, hashA, hashB, scan, qx, qy, qo, bpairs,
         border, bnext, bfront, keep, wtiles;
-    unsigned long long *h_res = nullptr; // pinned result block
-    size_t h_res_cap = 0;
+    char *h_ctl = nullptr; // pinned image of a tile launch's control block
+    size_t h_ctl_cap = 0;
+    bool slots_used = false; // every id in the slots is at most next_jid
+    uint32_t next_jid = 0;
     // pinned staging of short host strings (HostPacker): two halves, each busy
     // until its event
     char *h_stage = nullptr;
@@ -535,36 +537,43 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
     P.cls_p0[ncls] = pi;
     P.ncls = ncls;
     const int grid = cta;
+    const DevBuf slots0 = ctx->slots;
     if ((r = ensure(ctx, ctx->gf, sizeof(int32_t) * (size_t)std::max<int64_t>(gf_total, 1))) != ED_OK ||
-        (r = ensure(ctx, ctx->ctl, sizeof(LaunchCtl))) != ED_OK ||
-        (r = ensure(ctx, ctx->gctl, sizeof(GroupCtl) * ngroups)) != ED_OK ||
         (wide && (r = ensure(ctx, ctx->wtiles, sizeof(int32_t) * grid * lv_wide_tile_words((int)smax))) != ED_OK) ||
         (!wide && (r = ensure(ctx, ctx->slots, sizeof(JobSlot) * grid * JOB_RING)) != ED_OK) ||
-        (r = ensure(ctx, ctx->halo, sizeof(unsigned long long) * (size_t)grid * 4 * HMAX)) != ED_OK ||
-        (r = ensure(ctx, ctx->pdesc, sizeof(PairDesc) * np)) != ED_OK ||
-        (r = ensure(ctx, ctx->res, sizeof(unsigned long long) * R_COUNT * np)) != ED_OK)
+        (r = ensure(ctx, ctx->halo, sizeof(unsigned long long) * (size_t)grid * 4 * HMAX)) != ED_OK)
         return r;
-    const size_t hres = sizeof(unsigned long long) * R_COUNT * np + 64;
-    if (ctx->h_res_cap < hres) {
-        if (ctx->h_res)
-            cudaFreeHost(ctx->h_res);
-        ctx->h_res = nullptr;
-        ctx->h_res_cap = 0;
-        CK(cudaMallocHost((void **)&ctx->h_res, hres));
-        ctx->h_res_cap = hres;
+    // the launch's control words in one block, written by one copy and read
+    // back (from the launch's words on) by another: groups, pairs, launch,
+    // results
+    const size_t o_pairs = sizeof(GroupCtl) * ngroups;
+    const size_t o_ctl = (o_pairs + sizeof(PairDesc) * np + 63) & ~(size_t)63;
+    const size_t o_res = o_ctl + sizeof(LaunchCtl);
+    const size_t block = o_res + sizeof(unsigned long long) * R_COUNT * np;
+    if ((r = ensure(ctx, ctx->ctl, block)) != ED_OK)
+        return r;
+    if (ctx->h_ctl_cap < block) {
+        if (ctx->h_ctl)
+            cudaFreeHost(ctx->h_ctl);
+        ctx->h_ctl = nullptr;
+        ctx->h_ctl_cap = 0;
+        CK(cudaMallocHost((void **)&ctx->h_ctl, block));
+        ctx->h_ctl_cap = block;
     }
+    char *dctl = (char *)ctx->ctl.p;
+    std::memset(ctx->h_ctl, 0, block);
+    PairDesc *pd = (PairDesc *)(ctx->h_ctl + o_pairs);
+    LaunchCtl *hl = (LaunchCtl *)(ctx->h_ctl + o_ctl);
     // pair slot q runs job ord[q]; its counters land in row q
-    std::vector<PairDesc> pd(np);
     for (int q = 0; q < np; q++) {
         const TileJob &j = jobs[ord[q]];
-        pd[q] = PairDesc{};
         pd[q].A = j.A;
         pd[q].B = j.B;
         pd[q].n = j.n;
         pd[q].m = j.m;
         pd[q].TA = j.TA;
         pd[q].TB = j.TB;
-        pd[q].res = (unsigned long long *)ctx->res.p + (size_t)R_COUNT * q;
+        pd[q].res = (unsigned long long *)(dctl + o_res) + (size_t)R_COUNT * q;
         pd[q].dump = j.dump;
         pd[q].dump_tmax = (int32_t)j.dump_tmax;
         pd[q].keep = j.keep;
@@ -575,10 +584,10 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
         pd[q].init_t = j.init_t;
         pd[q].init_zero = j.init_zero;
     }
-    P.pairs = (const PairDesc *)ctx->pdesc.p;
+    P.pairs = (const PairDesc *)(dctl + o_pairs);
     P.npairs = np;
-    P.gctl = (GroupCtl *)ctx->gctl.p;
-    P.ctl = (LaunchCtl *)ctx->ctl.p;
+    P.gctl = (GroupCtl *)dctl;
+    P.ctl = (LaunchCtl *)(dctl + o_ctl);
     P.slots = (JobSlot *)ctx->slots.p;
     P.halo = (unsigned long long *)ctx->halo.p;
     P.gf = (int32_t *)ctx->gf.p;
@@ -603,38 +612,45 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
     P.stage = wide ? 0 : lv_tiles_smem_bytes((int)smax, h, 2) <= (size_t)ctx->smem_optin
                   ? 2
                   : (lv_tiles_smem_bytes((int)smax, h, 1) <= (size_t)ctx->smem_optin ? 1 : 0);
-    CK(cudaMemcpyAsync(ctx->pdesc.p, pd.data(), sizeof(PairDesc) * np, cudaMemcpyHostToDevice, s));
-    CK(cudaMemsetAsync(ctx->ctl.p, 0, sizeof(LaunchCtl), s));
-    CK(cudaMemsetAsync(ctx->gctl.p, 0, sizeof(GroupCtl) * ngroups, s));
-    if (!wide)
-        CK(cudaMemsetAsync(ctx->slots.p, 0, sizeof(JobSlot) * grid * JOB_RING, s));
-    CK(cudaMemsetAsync(ctx->res.p, 0, sizeof(unsigned long long) * R_COUNT * np, s));
+    if (!wide) {
+        // job ids go on from the last launch's, so that the slots' old words
+        // (10 MB of them) need no clearing; they are cleared when new, when
+        // another call wrote them, after a failed launch and before ids run out
+        if (!ctx->slots_used || ctx->slots.p != slots0.p || ctx->slots.bytes != slots0.bytes ||
+            ctx->next_jid >= 1u << 30) {
+            CK(cudaMemsetAsync(ctx->slots.p, 0, ctx->slots.bytes, s));
+            ctx->next_jid = 0;
+        }
+        ctx->slots_used = false;
+        P.jid0 = ctx->next_jid;
+    }
+    CK(cudaMemcpyAsync(dctl, ctx->h_ctl, block, cudaMemcpyHostToDevice, s));
     CK(cudaEventRecord(ctx->ev0, s));
     CK(wide ? launch_lv_wide(P, grid, s) : launch_lv_tiles(P, grid, s));
     CK(cudaEventRecord(ctx->ev1, s));
-    CK(cudaMemcpyAsync(ctx->h_res, ctx->res.p, sizeof(unsigned long long) * R_COUNT * np,
-                       cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync(ctx->h_res + (size_t)R_COUNT * np, ctx->ctl.p, sizeof(uint32_t),
-                       cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(hl, dctl + o_ctl, block - o_ctl, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     ctx->last.kernel_launches += 1;
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1);
     ctx->last.kernel_ms += ms;
-    const int lst = status_from_kernel(*(uint32_t *)(ctx->h_res + (size_t)R_COUNT * np));
+    const int lst = status_from_kernel(hl->error);
     if (lst != ED_OK) {
-        unsigned long long dg[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        cudaMemcpy(dg, (char *)ctx->ctl.p + offsetof(LaunchCtl, diag), sizeof(dg), cudaMemcpyDeviceToHost);
+        const unsigned long long *dg = hl->diag;
         char buf[256];
         std::snprintf(buf, sizeof(buf), "kernel check failed: site %llu cta %llu t %llu want %llx seen %llx %llx %llx",
                       dg[0], dg[1], dg[2], dg[3], dg[4], dg[5], dg[6]);
         ctx->last_err = buf;
         return lst;
     }
+    if (!wide) {
+        ctx->slots_used = true;
+        ctx->next_jid = std::max(ctx->next_jid, hl->last_jid);
+    }
     out.assign(np, TileOut{});
     for (int q = 0; q < np; q++) {
         const int i = ord[q];
-        const unsigned long long *R = ctx->h_res + (size_t)R_COUNT * q;
+        const unsigned long long *R = (const unsigned long long *)(ctx->h_ctl + o_res) + (size_t)R_COUNT * q;
         TileOut &o = out[i];
         o.st = (uint32_t)R[R_STATUS];
         const int64_t from = jobs[i].t0 > 0 ? jobs[i].t0 : jobs[i].init ? jobs[i].init_t : 0; // first round run
@@ -873,15 +889,15 @@ int ed_destroy(ed_ctx *ctx)
     engine_stop(ctx);
     cudaSetDevice(ctx->device);
     cudaStreamSynchronize(ctx->stream);
-    DevBuf *bufs[] = {&ctx->strA,  &ctx->strB,   &ctx->gf,    &ctx->ctl,    &ctx->gctl,      &ctx->slots,
-                      &ctx->halo,  &ctx->pdesc,  &ctx->res,   &ctx->dump,   &ctx->hashA,     &ctx->hashB,
+    DevBuf *bufs[] = {&ctx->strA,  &ctx->strB,   &ctx->gf,    &ctx->ctl,    &ctx->slots,
+                      &ctx->halo,  &ctx->pdesc,  &ctx->dump,   &ctx->hashA,     &ctx->hashB,
                       &ctx->scan,  &ctx->qx,     &ctx->qy,    &ctx->qo,     &ctx->bpairs,    &ctx->border,
                       &ctx->bnext, &ctx->bfront, &ctx->arena_buf, &ctx->s_pairs, &ctx->s_order, &ctx->s_next,
                       &ctx->keep,  &ctx->wtiles};
     for (DevBuf *b : bufs)
         release(ctx, *b);
-    if (ctx->h_res)
-        cudaFreeHost(ctx->h_res);
+    if (ctx->h_ctl)
+        cudaFreeHost(ctx->h_ctl);
     if (ctx->h_stage)
         cudaFreeHost(ctx->h_stage);
     for (cudaEvent_t e : ctx->stage_ev)
@@ -1136,6 +1152,7 @@ int ed_lcp_dev(ed_ctx *ctx, const uint8_t *A, size_t n, const uint8_t *B, size_t
         // one job per query (job id 1, pair 0 of a one-entry pair table)
         if (n >= (1ull << 31) || m >= (1ull << 31))
             return ED_EINVAL;
+        ctx->slots_used = false; // (the next tile launch clears them)
         if ((r = ensure(ctx, ctx->slots, sizeof(JobSlot) * q)) != ED_OK ||
             (r = ensure(ctx, ctx->pdesc, sizeof(PairDesc))) != ED_OK)
             return r;

@@ -81,7 +81,8 @@ struct __align__(64) GroupCtl {
 struct __align__(64) LaunchCtl {
     uint32_t error;
     uint32_t queue[MAX_CLS];   // next pair of each class's queue
-    uint32_t pad[3];
+    uint32_t last_jid;         // the largest job id a slot reached
+    uint32_t pad[2];
     // where the first failed wait gave up: site, CTA, round, awaited value,
     // values seen, done_k
     unsigned long long diag[8];
@@ -123,6 +124,7 @@ struct LvArgs {
     GroupCtl *gctl;
     LaunchCtl *ctl;
     JobSlot *slots;       // gridDim.x * JOB_RING slots (CTA c owns c * JOB_RING ..)
+    uint32_t jid0;        // this launch's job ids lie above this, every id left in the slots at or below it
     // tile edges: [gridDim.x][2 parity][2 sides][HMAX] words (round << 32) | L
     unsigned long long *halo;
     int32_t *gf;

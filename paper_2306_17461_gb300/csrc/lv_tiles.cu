@@ -373,7 +373,13 @@ struct Smem {
 //   result  = (jid << 32) | ~best  (so that red.max keeps the least offset)
 constexpr uint32_t NOMIS = 0xffffffffu;
 
-__device__ __forceinline__ bool claim_valid(unsigned long long w) { return (w >> 32) != 0; }
+// A claim on a word that no job of this launch wrote (ids up to jid0: the
+// slot has not been used in this launch, or its claim word is still on its
+// way) is nobody's: those jobs' strings and pair table are gone.
+__device__ __forceinline__ bool claim_valid(const LvArgs &P, unsigned long long w)
+{
+    return (uint32_t)(w >> 32) > P.jid0;
+}
 
 __device__ __forceinline__ void red_max_u64(unsigned long long *p, unsigned long long v)
 {
@@ -559,7 +565,7 @@ __device__ int claim_loop(const LvArgs &P, const Smem S, JobSlot *sl, int s, uns
     for (;;) {
         if (tid == 0) {
             const bool ready = wake && wake_ready(wake);
-            const int valid = claim_valid(w) ? 1 : 0;
+            const int valid = claim_valid(P, w) ? 1 : 0;
             const int go = valid ? claim_go(P, S, sl, s, w, best) : 0;
             S.bc()[0] = valid;
             S.bc()[3] = go;
@@ -613,7 +619,7 @@ __device__ int claim_loop2(const LvArgs &P, const Smem S, JobSlot *sl, int s, in
         const int sn = ps ^ 1;   // the stage for the claim resolved this turn
         if (tid == 0) {
             // 1. the claim in flight: valid, worth a scan?
-            const int nv = wn && claim_valid(wn) ? 1 : 0;
+            const int nv = wn && claim_valid(P, wn) ? 1 : 0;
             const int ng = nv ? claim_go(P, S, sl, s, wn, bestn, made + pvalid == 0 ? pre : nullptr) : 0;
             const unsigned long long wc = wn;
             // 2. its copies, in flight while the pending chunk is compared
@@ -1932,7 +1938,7 @@ __global__ void __launch_bounds__(CTA_THREADS, 1) lv_tiles_kernel(LvArgs P)
         S.jd()->pq = -1;
         *S.jring() = 0;
         for (int i = 0; i < JOB_RING; i++)
-            S.jids()[i] = 0;
+            S.jids()[i] = (int)P.jid0;
         for (int i = 0; i < 4; i++)
             S.tm()[i] = 0;
         *S.lone() = 0;
@@ -1994,6 +2000,9 @@ __global__ void __launch_bounds__(CTA_THREADS, 1) lv_tiles_kernel(LvArgs P)
         if (!group_sync(P, gc, G, S))
             break;
     }
+    if (threadIdx.x == 0)
+        for (int i = 0; i < JOB_RING; i++)
+            atomicMax(&P.ctl->last_jid, (uint32_t)S.jids()[i]);
 }
 
 cudaError_t launch_lv_tiles(const LvArgs &P, int grid, cudaStream_t s)
