@@ -410,201 +410,125 @@ __device__ __forceinline__ int64_t cta_scan(const uint8_t *A, int64_t n, const u
 }
 
 // ------------------------------------------------------- CTA sweep
-// An aligned 16-byte block loaded past the L1 (the bytes of a long slide are
-// read once; the L1 keeps the lines the rounds' start rows reuse).
-__device__ __forceinline__ uint4 ld_stream16(uintptr_t p)
+// An aligned 16-byte block.
+__device__ __forceinline__ uint4 ld_block(uintptr_t p) { return __ldg(reinterpret_cast<const uint4 *>(p)); }
+
+// Word i of the 16 bytes that start s8 / 8 bytes into word K of the run v.
+template <int K>
+__device__ __forceinline__ uint4 words_at(const uint32_t (&v)[8], uint32_t s8)
 {
-    uint4 v;
-    asm("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-        : "l"(p));
-    return v;
+    return make_uint4(__funnelshift_r(v[K], v[K + 1], s8), __funnelshift_r(v[K + 1], v[K + 2], s8),
+                      __funnelshift_r(v[K + 2], v[K + 3], s8), __funnelshift_r(v[K + 3], v[(K + 4) & 7], s8));
 }
 
-// The aligned block at blk if it overlaps [base, base + len) (len > 0),
-// else the block holding the string's first or last byte: a block that
-// overlaps the string lies in the same page as a valid byte and cannot
-// fault.  Bytes outside the window a caller asked for are masked by it.
-__device__ __forceinline__ uintptr_t safe_blk(uintptr_t base, int64_t len, uintptr_t blk)
+// The first differing byte of d = a ^ b, 16 bytes at string offsets o0 ..
+// o0 + 15, that lies in [0, len): its offset, or -1.
+__device__ __forceinline__ int64_t first_in(uint4 d, int64_t o0, int64_t len)
 {
-    const uintptr_t first = base & ~(uintptr_t)15, last = (base + (uintptr_t)len - 1) & ~(uintptr_t)15;
-    return blk < first ? first : (blk > last ? last : blk);
+    uint64_t d0 = ((uint64_t)d.y << 32) | d.x, d1 = ((uint64_t)d.w << 32) | d.z;
+    if (o0 < 0) { // (only the first block: bytes before the start)
+        const int skip = (int)-o0;
+        d0 &= skip >= 8 ? 0ull : ~0ull << (8 * skip);
+        d1 &= skip <= 8 ? ~0ull : ~0ull << (8 * (skip - 8));
+    }
+    const int i = d0 ? (__ffsll((long long)d0) - 1) >> 3 : d1 ? 8 + ((__ffsll((long long)d1) - 1) >> 3) : 16;
+    return i < 16 && o0 + i < len ? o0 + i : -1;
 }
 
-// The calling CTA compares A[x0 .. x0+len) with B[y0 .. y0+len) for
-// len <= blockDim.x * 16 * U - 16 (the blocks start up to 15 bytes before the
-// bytes compared) and returns the first mismatching offset, or -1.  Needs
-// x0 + len <= n and y0 + len <= m.  Every load is issued before the first
-// compare: one memory round trip per call.
+// The calling CTA compares A[x0 .. x0+len) with B[y0 ..) for any len > 0 (x0 +
+// len <= n, y0 + len <= m), blockDim.x * 16 * U bytes of each string a step
+// (4 KiB at 256 threads, U = 1), the next step's loads in flight while one
+// is compared, all in registers.  Returns the first mismatching offset, or -1.
+// Every thread must call it; s_min is a shared 64-bit scratch word.
 //
 // The A side is read in aligned 16-byte blocks: block j starts sa bytes
 // before A[x0] (sa = the misalignment of A + x0) and holds offsets
 // 16j - sa .. 16j - sa + 15.  The B bytes paired with them are bytes
 // qb .. qb + 15 of the 32-byte run made of B's aligned blocks j and j + 1
-// (counted from the block holding B[y0 - sa]); block j + 1 belongs to the
-// next lane, so it comes by shuffle (lane 31 takes the next row of blocks,
-// or one extra load after the last).  Warp w reads 32 * U consecutive
-// blocks.  Every thread must call it; s_min is a shared 64-bit scratch word.
-template <int U>
-__device__ __forceinline__ int64_t sweep_scan(const uint8_t *A, int64_t n, const uint8_t *B, int64_t m, int64_t x0,
-                                              int64_t y0, int64_t len, unsigned long long *s_min)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0)
-        *s_min = ~0ull;
-    const uintptr_t pa = (uintptr_t)(A + x0);
-    const uint32_t sa = (uint32_t)(pa & 15);
-    const uintptr_t a0 = pa - sa;
-    const uintptr_t pbs = (uintptr_t)(B + y0) - sa; // B address paired with a0
-    const uint32_t qb = (uint32_t)(pbs & 15);
-    const uintptr_t b0 = pbs - qb;
-    const uintptr_t Ab = (uintptr_t)A, Bb = (uintptr_t)B;
-    const int64_t jw = (int64_t)warp * 32 * U; // this warp's first block
-    uint4 va[U], vb[U];
-#pragma unroll
-    for (int u = 0; u < U; u++) {
-        const int64_t j = jw + u * 32 + lane;
-        va[u] = ld_stream16(safe_blk(Ab, n, a0 + 16 * j));
-        vb[u] = ld_stream16(safe_blk(Bb, m, b0 + 16 * j));
-    }
-    const uint4 vx = ld_stream16(safe_blk(Bb, m, b0 + 16 * (jw + 32 * U)));
-    int64_t best = -1;
-#pragma unroll
-    for (int u = 0; u < U; u++) {
-        // the B block after this lane's: the next lane's, or for lane 31 the
-        // first of the next row (the extra block after the last row)
-        const uint4 nb = u + 1 < U ? vb[u + 1] : vx;
-        uint4 nx;
-        nx.x = __shfl_down_sync(0xffffffffu, vb[u].x, 1);
-        nx.y = __shfl_down_sync(0xffffffffu, vb[u].y, 1);
-        nx.z = __shfl_down_sync(0xffffffffu, vb[u].z, 1);
-        nx.w = __shfl_down_sync(0xffffffffu, vb[u].w, 1);
-        const uint4 f0 = make_uint4(__shfl_sync(0xffffffffu, nb.x, 0), __shfl_sync(0xffffffffu, nb.y, 0),
-                                    __shfl_sync(0xffffffffu, nb.z, 0), __shfl_sync(0xffffffffu, nb.w, 0));
-        if (lane == 31)
-            nx = f0;
-        const uint4 bs = shift_bytes(vb[u], nx, qb);
-        const int64_t j = jw + u * 32 + lane;
-        // valid bytes of this block: offsets 16j - sa + i in [0, len)
-        const int64_t o0 = 16 * j - (int64_t)sa;
-        const int lo = o0 < 0 ? (int)-o0 : 0;
-        const int64_t hi64 = len - o0;
-        const int hi = hi64 >= 16 ? 16 : (hi64 <= 0 ? 0 : (int)hi64);
-        if (best < 0 && lo < hi) {
-            uint64_t d0 = ((uint64_t)(va[u].y ^ bs.y) << 32) | (uint64_t)(va[u].x ^ bs.x);
-            uint64_t d1 = ((uint64_t)(va[u].w ^ bs.w) << 32) | (uint64_t)(va[u].z ^ bs.z);
-            // keep bytes lo .. hi-1
-            const uint64_t k0lo = lo >= 8 ? 0ull : (~0ull << (8 * lo));
-            const uint64_t k1lo = lo <= 8 ? ~0ull : (~0ull << (8 * (lo - 8)));
-            const uint64_t k0hi = hi >= 8 ? ~0ull : ((1ull << (8 * hi)) - 1ull);
-            const uint64_t k1hi = hi <= 8 ? 0ull : (hi >= 16 ? ~0ull : ((1ull << (8 * (hi - 8))) - 1ull));
-            d0 &= k0lo & k0hi;
-            d1 &= k1lo & k1hi;
-            if (d0)
-                best = o0 + ((__ffsll((long long)d0) - 1) >> 3);
-            else if (d1)
-                best = o0 + 8 + ((__ffsll((long long)d1) - 1) >> 3);
-        }
-    }
-    if (__syncthreads_or(best >= 0)) {
-        if (best >= 0)
-            atomicMin(s_min, (unsigned long long)best);
-        __syncthreads();
-        const int64_t r = (int64_t)*s_min;
-        __syncthreads(); // read by all before the next call resets it
-        return r;
-    }
-    return -1;
-}
-
-// The calling CTA compares A[x0 .. x0+len) with B[y0 ..) for any len (x0 +
-// len <= n, y0 + len <= m), blockDim.x * 16 * U bytes of each string a step
-// (32 KiB at 256 threads, U = 8), the next step's loads in flight while one
-// is compared, all in registers.  Returns the first mismatching offset, or -1.
-// The blocks are sweep_scan's.  10^4 bytes take about 3 thousand cycles.  Every
-// thread must call it; s_min is a shared 64-bit scratch word, and the caller
-// meets a barrier before the next use.
+// (counted from the block holding B[y0 - sa]); the words of block j + 1 belong
+// to the next lane, so they come by shuffle (lane 31 takes the next row of
+// blocks, or one extra load after the last).  Warp w reads 32 * U consecutive
+// blocks a step; a block past the strings' ends is read at the end instead
+// (and the first of B's at its start).
+//
+// What bounds a short run is one round trip to L2 and the instructions around
+// it (asking for the next run's lines ahead gained nothing).  So the whole word
+// of the shift, qb / 4, is a template argument (uniform, and the same for all
+// slides of a diagonal), the clamps are on 32-bit block numbers, and bytes are
+// located only where words differ; a step of one block a thread is taken, the
+// loads allocate in L1 (the next round starts in these lines), and the callers
+// keep their registers (with U = 2 the kernel spills 580 bytes, with U = 4 it is
+// twice as slow).  Slides of 10^4 bytes: 3.9 -> 3.4 thousand cycles, 10^3 bytes:
+// 2.2 thousand.
 template <int U>
 struct SweepStep {
     uint4 a[U], b[U], x;
 };
+struct Sweep {
+    uintptr_t a0, b0;             // the blocks numbered 0
+    int32_t lastA, firstB, lastB; // the strings' own blocks
+    uint32_t sa, s8;
+};
 template <int U>
-__device__ __forceinline__ void sweep_load(SweepStep<U> &s, uintptr_t A, int64_t n, uintptr_t B, int64_t m,
-                                           uintptr_t a0, uintptr_t b0, int64_t j0)
+__device__ __forceinline__ void sweep_load(SweepStep<U> &s, const Sweep &W, int32_t j)
 {
-    const int lane = threadIdx.x & 31;
+    const int32_t l = j + (int32_t)(threadIdx.x & 31);
 #pragma unroll
     for (int u = 0; u < U; u++) {
-        s.a[u] = ld_stream16(safe_blk(A, n, a0 + 16 * (j0 + u * 32 + lane)));
-        s.b[u] = ld_stream16(safe_blk(B, m, b0 + 16 * (j0 + u * 32 + lane)));
+        s.a[u] = ld_block(W.a0 + 16 * (int64_t)min(l + u * 32, W.lastA));
+        s.b[u] = ld_block(W.b0 + 16 * (int64_t)max(min(l + u * 32, W.lastB), W.firstB));
     }
-    s.x = ld_stream16(safe_blk(B, m, b0 + 16 * (j0 + 32 * U)));
+    s.x = ld_block(W.b0 + 16 * (int64_t)max(min(j + 32 * U, W.lastB), W.firstB));
 }
 // The first mismatching offset of the thread's blocks, or -1.
-template <int U>
-__device__ __forceinline__ int64_t sweep_compare(const SweepStep<U> &s, uint32_t sa, uint32_t qb, int64_t j0,
-                                                 int64_t len)
+template <int U, int K>
+__device__ __forceinline__ int64_t sweep_compare(const SweepStep<U> &s, const Sweep &W, int32_t j, int64_t len)
 {
     const int lane = threadIdx.x & 31;
-    int64_t best = -1;
+    uint4 d[U];
+    uint32_t any = 0;
 #pragma unroll
     for (int u = 0; u < U; u++) {
         const uint4 nb = u + 1 < U ? s.b[u + 1 < U ? u + 1 : 0] : s.x;
-        uint4 nx; // the B block after this lane's
-        nx.x = __shfl_sync(0xffffffffu, lane == 0 ? nb.x : s.b[u].x, (lane + 1) & 31);
-        nx.y = __shfl_sync(0xffffffffu, lane == 0 ? nb.y : s.b[u].y, (lane + 1) & 31);
-        nx.z = __shfl_sync(0xffffffffu, lane == 0 ? nb.z : s.b[u].z, (lane + 1) & 31);
-        nx.w = __shfl_sync(0xffffffffu, lane == 0 ? nb.w : s.b[u].w, (lane + 1) & 31);
-        const uint4 bs = shift_bytes(s.b[u], nx, qb);
-        if (best < 0 && ((s.a[u].x ^ bs.x) | (s.a[u].y ^ bs.y) | (s.a[u].z ^ bs.z) | (s.a[u].w ^ bs.w))) {
-            // the first differing byte inside [0, len): offsets o0 + i
-            const int64_t o0 = 16 * (j0 + u * 32 + lane) - (int64_t)sa;
-            uint64_t d0 = ((uint64_t)(s.a[u].y ^ bs.y) << 32) | (s.a[u].x ^ bs.x);
-            uint64_t d1 = ((uint64_t)(s.a[u].w ^ bs.w) << 32) | (s.a[u].z ^ bs.z);
-            if (o0 < 0) { // (only the first block: sa bytes before the start)
-                const int skip = (int)-o0;
-                d0 &= skip >= 8 ? 0ull : ~0ull << (8 * skip);
-                d1 &= skip <= 8 ? ~0ull : ~0ull << (8 * (skip - 8));
-            }
-            int i = 16;
-            if (d0)
-                i = (__ffsll((long long)d0) - 1) >> 3;
-            else if (d1)
-                i = 8 + ((__ffsll((long long)d1) - 1) >> 3);
-            if (i < 16 && o0 + i < len)
-                best = o0 + i;
-        }
+        uint32_t v[8] = {s.b[u].x, s.b[u].y, s.b[u].z, s.b[u].w, 0, 0, 0, 0};
+        const uint32_t z[4] = {nb.x, nb.y, nb.z, nb.w};
+#pragma unroll
+        for (int i = 0; i <= K; i++) // (the next block's words up to K are in the run)
+            v[4 + i] = __shfl_sync(0xffffffffu, lane == 0 ? z[i] : v[i], (lane + 1) & 31);
+        const uint4 b = words_at<K>(v, W.s8);
+        d[u] = make_uint4(s.a[u].x ^ b.x, s.a[u].y ^ b.y, s.a[u].z ^ b.z, s.a[u].w ^ b.w);
+        any |= d[u].x | d[u].y | d[u].z | d[u].w;
+    }
+    int64_t best = -1;
+    if (any) {
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (best < 0)
+                best = first_in(d[u], 16 * ((int64_t)j + u * 32 + lane) - (int64_t)W.sa, len);
     }
     return best;
 }
-template <int U>
-__device__ __noinline__ int64_t stream_sweep(const uint8_t *A, int64_t n, const uint8_t *B, int64_t m, int64_t x0,
-                                             int64_t y0, int64_t len, unsigned long long *s_min)
+template <int U, int K>
+__device__ __forceinline__ int64_t sweep_run(const Sweep &W, int64_t len, unsigned long long *s_min)
 {
-    const uintptr_t pa = (uintptr_t)(A + x0), pb = (uintptr_t)(B + y0);
-    const uint32_t sa = (uint32_t)(pa & 15), qb = (uint32_t)((pb - sa) & 15);
-    const uintptr_t a0 = pa - sa, b0 = pb - sa - qb;
-    const uintptr_t Ab = (uintptr_t)A, Bb = (uintptr_t)B;
-    const int64_t nblk = ((int64_t)sa + len + 15) >> 4, step = (int64_t)(blockDim.x >> 5) * 32 * U;
-    int64_t j = (int64_t)(threadIdx.x >> 5) * 32 * U; // this warp's first block
-    if (threadIdx.x == 0)
-        *s_min = ~0ull;
+    const int32_t nblk = (int32_t)(((int64_t)W.sa + len + 15) >> 4), step = (int32_t)(blockDim.x >> 5) * 32 * U;
+    int32_t j = (int32_t)(threadIdx.x >> 5) * 32 * U; // this warp's first block
     SweepStep<U> s0, s1;
-    sweep_load(s0, Ab, n, Bb, m, a0, b0, j);
-    for (int64_t at = 0;;) {
+    sweep_load(s0, W, j);
+    for (int32_t at = 0;;) {
         // two steps a turn, so that each buffer stays in its registers
         int64_t best;
         const bool more1 = at + step < nblk;
         if (more1)
-            sweep_load(s1, Ab, n, Bb, m, a0, b0, j + step);
-        best = sweep_compare(s0, sa, qb, j, len);
+            sweep_load(s1, W, j + step);
+        best = sweep_compare<U, K>(s0, W, j, len);
         at += step;
         j += step;
         bool hit = __syncthreads_or(best >= 0) != 0;
         if (!hit && more1) {
             if (at + step < nblk)
-                sweep_load(s0, Ab, n, Bb, m, a0, b0, j + step);
-            best = sweep_compare(s1, sa, qb, j, len);
+                sweep_load(s0, W, j + step);
+            best = sweep_compare<U, K>(s1, W, j, len);
             at += step;
             j += step;
             hit = __syncthreads_or(best >= 0) != 0;
@@ -613,10 +537,35 @@ __device__ __noinline__ int64_t stream_sweep(const uint8_t *A, int64_t n, const 
             if (best >= 0)
                 atomicMin(s_min, (unsigned long long)best);
             __syncthreads();
-            return (int64_t)*s_min; // (the caller meets a barrier before the next use)
+            const int64_t r = (int64_t)*s_min;
+            __syncthreads(); // read by all before the next call resets it
+            return r;
         }
         if (at >= nblk)
             return -1;
+    }
+}
+template <int U>
+__device__ __noinline__ int64_t stream_sweep(const uint8_t *A, int64_t n, const uint8_t *B, int64_t m, int64_t x0,
+                                             int64_t y0, int64_t len, unsigned long long *s_min)
+{
+    const uintptr_t pa = (uintptr_t)(A + x0), pb = (uintptr_t)(B + y0);
+    Sweep W;
+    W.sa = (uint32_t)(pa & 15);
+    const uint32_t qb = (uint32_t)((pb - W.sa) & 15);
+    W.s8 = (qb & 3) * 8;
+    W.a0 = pa - W.sa;
+    W.b0 = pb - W.sa - qb;
+    W.lastA = (int32_t)(((int64_t)((uintptr_t)(A + n - 1) - W.a0)) >> 4);
+    W.firstB = (int32_t)(((int64_t)(((uintptr_t)B & ~(uintptr_t)15) - W.b0)) >> 4);
+    W.lastB = (int32_t)(((int64_t)((uintptr_t)(B + m - 1) - W.b0)) >> 4);
+    if (threadIdx.x == 0)
+        *s_min = ~0ull;
+    switch (qb >> 2) {
+    case 0: return sweep_run<U, 0>(W, len, s_min);
+    case 1: return sweep_run<U, 1>(W, len, s_min);
+    case 2: return sweep_run<U, 2>(W, len, s_min);
+    default: return sweep_run<U, 3>(W, len, s_min);
     }
 }
 
@@ -762,34 +711,33 @@ __device__ __forceinline__ bool stage_wait(const Stage T, uint64_t spin_ns, uint
 // The stage is released (phase passed, reads ordered before later bulk
 // copies into it) before the result is combined.  s_min: a shared 64-bit
 // scratch word.
-__device__ __forceinline__ int64_t stage_compare(const Stage T, const StagedChunk K, unsigned long long *s_min)
+template <int K>
+__device__ __forceinline__ int64_t stage_first(const Stage T, const StagedChunk C)
 {
-    const int tid = threadIdx.x;
-    int64_t best = -1;
-    for (int64_t j = tid; j < K.nblk && best < 0; j += blockDim.x) {
+    const uint32_t s8 = (C.qb & 3) * 8;
+    for (int64_t j = threadIdx.x; j < C.nblk; j += blockDim.x) {
         const uint4 va = *reinterpret_cast<const uint4 *>(T.a + 16 * j);
         const uint4 lo = *reinterpret_cast<const uint4 *>(T.b + 16 * j);
         const uint4 hi = *reinterpret_cast<const uint4 *>(T.b + 16 * j + 16);
-        const uint4 bs = shift_bytes(lo, hi, K.qb);
-        const int64_t o0 = 16 * j - (int64_t)K.sa;
-        const int lo_i = o0 < 0 ? (int)-o0 : 0;
-        const int64_t hi64 = K.len - o0;
-        const int hi_i = hi64 >= 16 ? 16 : (hi64 <= 0 ? 0 : (int)hi64);
-        if (lo_i < hi_i) {
-            uint64_t d0 = ((uint64_t)(va.y ^ bs.y) << 32) | (uint64_t)(va.x ^ bs.x);
-            uint64_t d1 = ((uint64_t)(va.w ^ bs.w) << 32) | (uint64_t)(va.z ^ bs.z);
-            const uint64_t k0lo = lo_i >= 8 ? 0ull : (~0ull << (8 * lo_i));
-            const uint64_t k1lo = lo_i <= 8 ? ~0ull : (~0ull << (8 * (lo_i - 8)));
-            const uint64_t k0hi = hi_i >= 8 ? ~0ull : ((1ull << (8 * hi_i)) - 1ull);
-            const uint64_t k1hi = hi_i <= 8 ? 0ull : (hi_i >= 16 ? ~0ull : ((1ull << (8 * (hi_i - 8))) - 1ull));
-            d0 &= k0lo & k0hi;
-            d1 &= k1lo & k1hi;
-            if (d0)
-                best = o0 + ((__ffsll((long long)d0) - 1) >> 3);
-            else if (d1)
-                best = o0 + 8 + ((__ffsll((long long)d1) - 1) >> 3);
+        const uint32_t v[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+        const uint4 b = words_at<K>(v, s8);
+        const uint4 d = make_uint4(va.x ^ b.x, va.y ^ b.y, va.z ^ b.z, va.w ^ b.w);
+        if (d.x | d.y | d.z | d.w) {
+            const int64_t r = first_in(d, 16 * j - (int64_t)C.sa, C.len);
+            if (r >= 0)
+                return r;
         }
     }
+    return -1;
+}
+static __device__ __noinline__ int64_t stage_compare(const Stage T, const StagedChunk K, unsigned long long *s_min)
+{
+    const int tid = threadIdx.x;
+    const uint32_t q = K.qb >> 2;
+    const int64_t best = q == 0   ? stage_first<0>(T, K)
+                         : q == 1 ? stage_first<1>(T, K)
+                         : q == 2 ? stage_first<2>(T, K)
+                                  : stage_first<3>(T, K);
     fence_proxy_async_smem();
     if (tid == 0)
         *s_min = ~0ull;

@@ -335,7 +335,6 @@ struct Smem {
     __device__ __forceinline__ int *left() const { return at<int>(144); }
     __device__ __forceinline__ int *kf() const { return at<int>(152); } // the target row was n in the round before
     __device__ __forceinline__ int *nR() const { return at<int>(156); }
-    __device__ __forceinline__ int *lone() const { return at<int>(176); } // lean_slides
     __device__ __forceinline__ unsigned long long *lead() const { return at<unsigned long long>(184); }
     __device__ __forceinline__ JobDesc *jd() const { return at<JobDesc>(192); } // the job last claimed from
     // cycles in rounds, open slides, halo waits and epoch changes (thread 0's)
@@ -490,8 +489,7 @@ __device__ __forceinline__ int claim_go(const LvArgs &P, const Smem S, JobSlot *
 
 // The first mismatch of A[x0..x0+len) vs B[y0..) (len <= CHUNK_BYTES), or
 // -1: by bulk copies into the CTA's stage when it has one, else (and for small
-// chunks) by register sweeps.  Whole CTA.  (A
-// stage wait that gave up has set the launch status; the chunk then counts as
+// chunks) by register sweeps.  Whole CTA.  (A stage wait that gave up has set the launch status; the chunk then counts as
 // equal and the launch reports the timeout.)
 __device__ __forceinline__ int64_t chunk_scan(const LvArgs &P, const Smem S, const uint8_t *A, int64_t n,
                                               const uint8_t *B, int64_t m, int64_t x0, int64_t y0, int64_t len)
@@ -502,16 +500,7 @@ __device__ __forceinline__ int64_t chunk_scan(const LvArgs &P, const Smem S, con
         const int64_t r = stage_scan<CHUNK_BYTES>(stage_of(S.stg()), A, n, B, m, x0, y0, len, S.smin(), P.spin_ns, &P.ctl->error);
         return r >= 0 ? r : -1;
     }
-    if (len <= SMALL_CHUNK)
-        return sweep_scan<1>(A, n, B, m, x0, y0, len, S.smin());
-    constexpr int U = CHUNK_BYTES / (CTA_THREADS * 16);
-    constexpr int64_t STEP = CTA_THREADS * 16 * U - 16;
-    for (int64_t o = 0; o < len; o += STEP) {
-        const int64_t r = sweep_scan<U>(A, n, B, m, x0 + o, y0 + o, min(STEP, len - o), S.smin());
-        if (r >= 0)
-            return o + r;
-    }
-    return -1;
+    return stream_sweep<1>(A, n, B, m, x0, y0, len, S.smin());
 }
 
 // The whole CTA scans claimed chunk c of job jid, cached in S.jd() (when go),
@@ -863,8 +852,8 @@ __device__ __noinline__ int64_t run_job(const LvArgs &P, const Smem S, const Pai
 // CTA streams up to ALONE_BYTES of each string itself (local_chunks chunks at
 // least); the rest, and the whole of a slide when they run longer, goes to
 // jobs of at most JOB_MAX_CHUNKS chunks each, helped by other CTAs.  A job
-// takes 14 to 20 thousand cycles however short its slide is; the CTA alone
-// takes 3 thousand for 10^4 bytes and as many as a job for about 10^5.
+// takes 10 thousand cycles for 10^5 bytes and 15 thousand for 2 * 10^6; the CTA
+// alone takes 3.4 thousand for 10^4 bytes and as many as a job for about 6 * 10^4.
 // Returns the first mismatch offset, or lim (every thread; a barrier lies
 // between two calls).
 constexpr int64_t ALONE_BYTES = 64 * 1024;
@@ -878,7 +867,7 @@ __device__ __noinline__ int64_t long_slide(const LvArgs &P, const Smem S, const 
                                       (int64_t)max(0, P.local_chunks) * CHUNK_BYTES));
     int64_t r = -1;
     if (loc > 0)
-        r = stream_sweep<2>(Q.A, Q.n, Q.B, Q.m, x0, y0, loc, S.smin());
+        r = stream_sweep<1>(Q.A, Q.n, Q.B, Q.m, x0, y0, loc, S.smin());
     int64_t off = loc;
     while (r < 0 && off < lim0) {
         // slides that run to a few hundred KB go in small chunks, one load a
@@ -1315,39 +1304,31 @@ __device__ __forceinline__ BlockOut run_block(const LvArgs &P, const Smem S, con
     return BlockOut{C.slide, C.mism, C.hashq, C.coll, C.longs, C.opens, kfound >= 0 ? 1 : 0};
 }
 
-// A lone slide this long is worth the whole CTA (one step of stream_sweep).
-constexpr int32_t LONE_BYTES = 2048;
-
-// The open slides of a lean round (out of line: most rounds have none):
-// one warp each, up to t2_cap bytes, then the whole CTA for those still
-// open -- or, for a lone slide after a lone one that outran its warp (or went
-// on for LONE_BYTES), the whole CTA at once.  Every thread calls it (after a barrier); the final
-// rows are visible to every thread when it returns.
+// The open slides of a lean round (out of line: most rounds have none): a
+// lone one goes to the whole CTA at once (it matched 21 bytes and more: the
+// alignment path's, nearly always, of n / k bytes; a warp's step first, up to
+// t2_cap bytes, cost 2 thousand cycles when it fell short and gained nothing
+// when it did not: n = 10^6, k = 500, slides of 2 KB, 1.88 -> 1.53 ms), several
+// to one warp each, then to the whole CTA those still open.  Every thread calls
+// it (after a barrier); the final rows are visible to every thread when it
+// returns.
 __device__ __forceinline__ void lean_slides(const LvArgs &P, const Smem S, const Pair Q, int32_t *cur, int64_t off,
                                          int32_t *Ld, const int32_t *Lc, int nlo, int64_t a, int64_t b, int pr,
                                          Counters &C)
 {
-    // lone: whether the CTA's last lone slide outran one warp (t2_cap bytes);
-    // the next lone one then goes to the whole CTA at once (its job opens
-    // without the warp's step first): on the alignment path, slides long
-    // and short come in runs
-    int *lone = S.lone();
-    const bool direct = nlo == 1 && *lone != 0;
-    if (direct && !Q.hash) {
+    if (nlo == 1 && !Q.hash) {
         const int64_t d = Ld[0], c = Lc[0], lim = min(Q.n - c, Q.m - c - d);
+        const bool own = d >= a && d < b;
         const int64_t rr = long_slide(P, S, Q, c, c + d, lim);
-        C.longs++;
+        C.longs += rr >= P.t2_cap;
         if (threadIdx.x < 32) {
             if (threadIdx.x == 0) {
-                cur[d - off] = (int32_t)finish_slide(Q, c, d, c + rr, c + lim, d >= a && d < b, C);
-                *lone = rr > LONE_BYTES;
+                cur[d - off] = (int32_t)finish_slide(Q, c, d, c + rr, c + lim, own, C);
+                C.opens += own;
             }
             prefetch_next(Q.A, Q.n, Q.B, Q.m, c + rr, c + rr + d);
         }
-        __syncthreads();
-        return;
-    }
-    if (direct) {
+    } else if (nlo == 1) {
         cta_slides(P, S, Q, cur, off, Ld, Lc, nlo, a, b, C);
     } else {
         const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -1355,11 +1336,8 @@ __device__ __forceinline__ void lean_slides(const LvArgs &P, const Smem S, const
         __syncthreads();
         if (S.left()[pr])
             cta_slides(P, S, Q, cur, off, Ld, Lc, nlo, a, b, C);
-    }
-    if (threadIdx.x == 0) {
-        if (nlo == 1)
-            *lone = direct ? (cur[Ld[0] - off] - Lc[0] > LONE_BYTES) : S.left()[pr];
-        S.left()[pr] = 0;
+        if (threadIdx.x == 0)
+            S.left()[pr] = 0;
     }
     __syncthreads();
 }
@@ -1941,7 +1919,6 @@ __global__ void __launch_bounds__(CTA_THREADS, 1) lv_tiles_kernel(LvArgs P)
             S.jids()[i] = (int)P.jid0;
         for (int i = 0; i < 4; i++)
             S.tm()[i] = 0;
-        *S.lone() = 0;
         for (int i = 0; S.stg() && i < P.stage; i++) {
             const Stage T = stage_of(S.stg() + i * STAGE_STRIDE);
             mbar_init(T.bar, 1);

@@ -252,6 +252,29 @@ def test_grid_lcp_at_chunk_ends(ctx, orc, method, sa, sy):
         assert got[0] == off, (method, sa, sy, off)
 
 
+@pytest.mark.parametrize("method", [2, 7])
+@pytest.mark.parametrize("sb", range(16))
+def test_grid_lcp_every_shift(ctx, orc, method, sb):
+    """Every byte shift between the strings, from start rows at every
+    alignment: mismatches in the first bytes, at the ends of a step of the
+    sweep (4096 bytes) and of the strings, and none."""
+    from paper_2306_17461_gb300 import binding as ed
+
+    n, d = 2 * 4096 + 37, 3
+    rng = np.random.default_rng(430 + sb)
+    A = rng.integers(0, 4, n, dtype=np.uint8)
+    dA = dev(A)
+    for off in [0, 1, 15, 16, 31, 4095, 4096, 4097, 8191, n - 2, n - 1, n]:
+        B = np.concatenate([rng.integers(0, 4, d, dtype=np.uint8), A])
+        if off < n:
+            B[off + d] ^= 1
+        dB = dev(np.concatenate([np.zeros(sb, np.uint8), B]))[sb:]
+        xs = np.array([x for x in [0, 1, 7, 15, 16, 17, off - 17, off - 3, off, off + 1, n - 1] if 0 <= x < n])
+        want = [(off if x <= off else n) - x for x in xs]
+        got = ed.ed_lcp_dev(ctx.h, dA, dB, xs, xs + d, method)
+        assert np.array_equal(got, want), (method, sb, off)
+
+
 @pytest.mark.parametrize("gap", [3000, 4080, 16 * 1024, 65_535, 65_537, 300_000, 1_100_000])
 def test_slide_lengths_across_the_paths(orc, gap):
     """Slides around the lengths at which they change hands: a warp, the CTA
