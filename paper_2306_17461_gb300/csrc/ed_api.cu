@@ -35,6 +35,15 @@ constexpr int64_t MAX_LEN = (1ll << 31) - 64;
 constexpr uint64_t Q61H = (1ull << 61) - 1;
 constexpr int BATCH_W = 4096; // band capacity of one batch CTA
 constexpr int START_TILE = 2048; // diagonals per CTA a single pair starts with
+// Single pairs of strings up to FEW_MAX bytes run on FEW_CTAS CTAs: one CTA
+// streams their slides as fast as others would help, their widest band is 171
+// diagonals a CTA, and the group's barriers, its skipping tiles and the end of
+// the pair wait for 24 CTAs instead of 152.  n = 10^3, k = 13: 95 -> 83 us a call,
+// k = 27: 105 -> 95 us, k = 80: 150 -> 133 us.  (On longer strings the same is
+// gained for k < 100, but a band of thousands of diagonals wants the whole
+// grid, and moving it there costs 100 us.  8 CTAs and fewer, 32 and more: slower.)
+constexpr int FEW_CTAS = 24;
+constexpr int64_t FEW_MAX = 2048;
 
 // host mod 2^61-1 (exact 128-bit product), for the hash base powers
 uint64_t hmul(uint64_t a, uint64_t b)
@@ -739,7 +748,8 @@ int run_pair(ed_ctx *ctx, const uint8_t *dA, int64_t n, const uint8_t *dB, int64
              cudaStream_t s, int32_t *dump, int64_t dump_tmax, uint64_t *k_out)
 {
     int r;
-    TileJob j{dA, dB, n, m, nullptr, nullptr, dump, dump_tmax, ctx->grid, 1.0};
+    const int G = std::max(n, m) <= FEW_MAX ? std::min(ctx->grid, FEW_CTAS) : ctx->grid;
+    TileJob j{dA, dB, n, m, nullptr, nullptr, dump, dump_tmax, G, 1.0};
     // narrow tiles first (a large L1), saved and resumed on wider ones when
     // the band outgrows them
     j.smax_want = START_TILE;

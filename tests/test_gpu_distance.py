@@ -219,3 +219,17 @@ def test_skew_lengthens_the_slides(ctxs):
         st = ctxs["default"].stats()
         means.append(st["slide_chars"] / st["extensions"])
     assert means[0] < means[1] < means[2], means
+
+
+@pytest.mark.parametrize("n,m", [(2047, 2048), (2048, 2048), (2048, 2049), (1, 2048), (0, 3)])
+def test_short_pairs_on_few_ctas(ctxs, orc, n, m):
+    """Pairs on either side of the length up to which the grid is not all
+    used, from a few edits to the widest band such strings can have."""
+    rng = np.random.default_rng(n + m)
+    A = rng.integers(0, 4, n, dtype=np.uint8)
+    near = np.concatenate([A, rng.integers(0, 4, max(0, m - n), dtype=np.uint8)])[:m]
+    near[:: max(1, m // 9)] ^= 1
+    for B in (near, rng.integers(0, 4, m, dtype=np.uint8), rng.integers(8, 12, m, dtype=np.uint8)):
+        want = orc.lv(A, B)
+        for name in ctxs:
+            assert ctxs[name].distance(A, B) == want, name
