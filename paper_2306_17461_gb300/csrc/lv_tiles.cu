@@ -585,7 +585,10 @@ __device__ int claim_loop(const LvArgs &P, const Smem S, JobSlot *sl, int s, uns
 // each claim's chunk is staged by bulk copies as soon as its claim word is
 // back, while the chunk claimed before it is compared, and the claim after
 // it is in flight meanwhile; so a helper has two chunks' bytes in flight.
-// The same claims, answers and stopping rules as claim_loop.
+// The same claims, answers and stopping rules as claim_loop, but a CTA with
+// nothing pending takes one small chunk only, and answers it at once: such jobs
+// are short, and a chunk queued behind another was their last answer (slides of
+// 10^5 bytes: 6.7 -> 6.0 us a round).
 __device__ int claim_loop2(const LvArgs &P, const Smem S, JobSlot *sl, int s, int budget, const Wake *wake)
 {
     const int tid = threadIdx.x;
@@ -620,7 +623,7 @@ __device__ int claim_loop2(const LvArgs &P, const Smem S, JobSlot *sl, int s, in
             }
             // 3. the claim after it, in flight meanwhile
             const bool ready = wake && wake_ready(wake);
-            const bool more = ng && !ready && made + pvalid + nv < budget;
+            const bool more = ng && !ready && made + pvalid + nv < (S.jd()->chunk > SMALL_CHUNK ? budget : 1);
             wn = more ? atomicAdd(&sl->claim, 1ull) : 0ull;
             bestn = more ? ld_relaxed_u64(&sl->result) : ~0ull;
             S.bc()[0] = nv;
@@ -632,6 +635,10 @@ __device__ int claim_loop2(const LvArgs &P, const Smem S, JobSlot *sl, int s, in
         const unsigned long long wcn = (unsigned long long)S.bcl()[0];
         const int64_t nc = (int64_t)(uint32_t)wcn;
         __syncthreads();
+        if (ng == 2 && !pvalid) { // a small chunk: swept and answered at once, no second one
+            scan_claim(P, S, sl, (uint32_t)(wcn >> 32), nc, 1);
+            return made + 1;
+        }
         // 4. the pending chunk: compared (when worth it) and answered
         if (pvalid) {
             int64_t r = -1;
