@@ -257,8 +257,8 @@ uint64_t ed_hash_base(ed_ctx *ctx);
  * looked up once per device ordinal in it).  base must lie in
  * [2, 2^61-2].  len above ED_NOALLOC_MAX_LEN returns ED_EINVAL.  The
  * first call on a device looks up the array's device address (make that
- * call before any stream capture).  Every call shares the array and clears
- * it on `stream` before use: calls whose work overlaps on the GPU (two
+ * call before any stream capture).  Every call shares the array and writes
+ * it on `stream` before reading it: calls whose work overlaps on the GPU (two
  * streams, or two threads) race and must be serialised by the caller.
  * Synchronous on `stream` (NULL = legacy default). */
 int ed_prefix_hash_noalloc(const uint8_t *X, size_t len, uint64_t base, uint64_t *T,

@@ -615,9 +615,8 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
     P.sync_rounds = 16 * h;
     P.help_div = ctx->eff.help_div;
     P.local_chunks = ctx->eff.local_chunks;
-    // bulk-copy staging of long-slide chunks (two stages: the owner streams
-    // its first chunks with the next one's copies in flight) when the tiles
-    // leave room for it
+    // bulk-copy staging of long-slide chunks (two stages: a helper's next
+    // chunk is on its way while one is compared) when the tiles leave room
     P.stage = wide ? 0 : lv_tiles_smem_bytes((int)smax, h, 2) <= (size_t)ctx->smem_optin
                   ? 2
                   : (lv_tiles_smem_bytes((int)smax, h, 1) <= (size_t)ctx->smem_optin ? 1 : 0);
@@ -872,7 +871,7 @@ int ed_create(ed_ctx **out, const ed_config *cfg)
     size_t fr = 0, tot = 0;
     CK(cudaMemGetInfo(&fr, &tot));
     c->budget = c->cfg.mem_budget_bytes ? c->cfg.mem_budget_bytes : (size_t)(fr * 0.6);
-    // co-resident grid for the cooperative tile kernel: one 512-thread CTA per SM
+    // co-resident grid for the cooperative tile kernel: one CTA per SM
     c->grid = c->cfg.grid_ctas > 0 ? std::min(c->cfg.grid_ctas, c->num_sms) : c->num_sms;
     c->grid = std::min(c->grid, MAX_GRID);
     c->wgrid = std::min(c->cfg.grid_ctas > 0 ? c->grid : WIDE_PER_SM * c->num_sms, MAX_GRID);

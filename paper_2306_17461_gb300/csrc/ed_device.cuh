@@ -41,11 +41,6 @@ __device__ __forceinline__ void st_release(uint32_t *p, uint32_t v)
 }
 __device__ __forceinline__ int32_t ld_cg(const int32_t *p) { return __ldcg(p); }
 __device__ __forceinline__ void st_cg(int32_t *p, int32_t v) { __stcg(p, v); }
-__device__ __forceinline__ int64_t ld_vol64(const int64_t *p)
-{
-    return *(const volatile int64_t *)p;
-}
-
 // ------------------------------------------------------- string windows
 // A 16-byte aligned block is loaded only if it overlaps the string
 // [base, base+len): such a block lies in the same page as a valid byte, so
@@ -165,114 +160,6 @@ __device__ __forceinline__ int64_t slide_thread_w(const uint8_t *A, int64_t n, c
         return lim;
     *open = true;
     return l;
-}
-
-// The word part of slide_thread_w alone: returns the matched length when
-// the words decide the slide (a mismatch within them, or lim reached), else
-// -1 with *avail = the bytes they showed equal.
-__device__ __forceinline__ int64_t word_slide(const uint8_t *A, const uint8_t *B, int64_t x, int64_t y,
-                                              int64_t lim, uint32_t wa, uint32_t wb, int64_t *avail)
-{
-    if (lim <= 0)
-        return 0;
-    const uint32_t sa = (uint32_t)((uintptr_t)(A + x) & 3), sb = (uint32_t)((uintptr_t)(B + y) & 3);
-    wa >>= 8 * sa;
-    wb >>= 8 * sb;
-    int64_t av = (int64_t)(4 - max(sa, sb));
-    if (av > lim)
-        av = lim;
-    const uint32_t mask = av >= 4 ? 0xffffffffu : ((1u << (8 * av)) - 1u);
-    const uint32_t dif = (wa ^ wb) & mask;
-    if (dif)
-        return (__ffs((int)dif) - 1) >> 3;
-    if (av >= lim)
-        return lim;
-    *avail = av;
-    return -1;
-}
-
-// The aligned 4-byte word holding A[x] and the one after it, and the same
-// for B[y]: at least five bytes from each start row whatever its
-// alignment.  The second word is loaded only while it still holds a byte of
-// the string (an aligned word holding a valid byte cannot fault); else 0.
-__device__ __forceinline__ void word_load2(const uint8_t *A, int64_t n, const uint8_t *B, int64_t m,
-                                           int64_t x, int64_t y, uint2 &wa, uint2 &wb)
-{
-    const uintptr_t pa = (uintptr_t)(A + x) & ~(uintptr_t)3, pb = (uintptr_t)(B + y) & ~(uintptr_t)3;
-    wa.x = __ldg(reinterpret_cast<const uint32_t *>(pa));
-    wb.x = __ldg(reinterpret_cast<const uint32_t *>(pb));
-    wa.y = pa + 4 < (uintptr_t)(A + n) ? __ldg(reinterpret_cast<const uint32_t *>(pa + 4)) : 0u;
-    wb.y = pb + 4 < (uintptr_t)(B + m) ? __ldg(reinterpret_cast<const uint32_t *>(pb + 4)) : 0u;
-}
-
-// The LCP from (x, y) as far as the words of word_load2 decide it: the
-// matched length when a mismatch shows within them or `lim` is reached,
-// else -1 (every byte they hold matched; the slide goes on elsewhere).
-__device__ __forceinline__ int64_t word_slide2(const uint8_t *A, const uint8_t *B, int64_t x, int64_t y,
-                                               int64_t lim, uint2 wa, uint2 wb)
-{
-    if (lim <= 0)
-        return 0;
-    const uint32_t sa = (uint32_t)((uintptr_t)(A + x) & 3), sb = (uint32_t)((uintptr_t)(B + y) & 3);
-    const uint64_t va = (((uint64_t)wa.y << 32) | wa.x) >> (8 * sa);
-    const uint64_t vb = (((uint64_t)wb.y << 32) | wb.x) >> (8 * sb);
-    int64_t av = (int64_t)(8 - max(sa, sb));
-    if (av > lim)
-        av = lim;
-    const uint64_t mask = av >= 8 ? ~0ull : ((1ull << (8 * av)) - 1ull);
-    const uint64_t dif = (va ^ vb) & mask;
-    if (dif)
-        return (__ffsll((long long)dif) - 1) >> 3;
-    return av >= lim ? lim : -1;
-}
-
-// The 16-byte window part of slide_thread_w, from l bytes already equal:
-// four windows (64 bytes) per step, their loads in flight together.
-static __device__ __noinline__ int64_t slide_more(const uint8_t *A, int64_t n, const uint8_t *B, int64_t m,
-                                           int64_t x, int64_t y, int64_t l, int64_t lim, int64_t cap,
-                                           bool *open)
-{
-    *open = false;
-    const int64_t stop = min(lim, cap);
-    while (l < stop) {
-        uint4 va[4], vb[4];
-#pragma unroll
-        for (int w = 0; w < 4; w++) {
-            if (l + 16 * w < stop) {
-                va[w] = load16(A, n, x + l + 16 * w);
-                vb[w] = load16(B, m, y + l + 16 * w);
-            }
-        }
-#pragma unroll
-        for (int w = 0; w < 4; w++) {
-            if (l + 16 * w < stop) {
-                const int f = first_diff16(va[w], vb[w]);
-                if (f < 16)
-                    return min(l + 16 * w + f, lim);
-            }
-        }
-        l = min(l + 64, stop);
-    }
-    if (l >= lim)
-        return lim;
-    *open = true;
-    return l;
-}
-
-// Asks L2 for len bytes of X from byte x on (clipped to the string), by the
-// copy engine: one bulk prefetch, no load issued by the calling thread.  It
-// covers whole 16-byte blocks, never past the one that holds the string's
-// last byte.
-__device__ __forceinline__ void bulk_prefetch_l2(const uint8_t *X, int64_t len_x, int64_t x, int64_t len)
-{
-    if (x < 0 || x >= len_x || len <= 0)
-        return;
-    const uintptr_t lo = (uintptr_t)(X + x) & ~(uintptr_t)15;
-    const uintptr_t end = ((uintptr_t)(X + len_x) + 15) & ~(uintptr_t)15;
-    const uintptr_t hi = min((((uintptr_t)(X + x) + (uintptr_t)len) + 15) & ~(uintptr_t)15, end);
-    uint64_t g;
-    asm("cvta.to.global.u64 %0, %1;" : "=l"(g) : "l"(lo));
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(g), "r"((uint32_t)(hi - lo)) : "memory");
 }
 
 // Slides at least this long are followed by a prefetch of what follows
@@ -768,50 +655,6 @@ __device__ __noinline__ int64_t stage_scan(const Stage T, const uint8_t *A, int6
     if (!stage_wait(T, spin_ns, err))
         return -2;
     return stage_compare(T, K, s_min);
-}
-
-// A[x0 .. x0+lim) against B[y0 ..) chunk by chunk through two stages, the
-// next chunk's copies in flight while the current one is compared.  Whole
-// CTA.  Returns the first mismatching offset, lim if none, or -2 when a
-// wait gave up (*err set).  Before returning it waits for the copies still
-// in flight, so that both stages are idle.
-template <int CH>
-__device__ __noinline__ int64_t stream_scan(const Stage T0, const Stage T1, const uint8_t *A, int64_t n,
-                                            const uint8_t *B, int64_t m, int64_t x0, int64_t y0, int64_t lim,
-                                            unsigned long long *s_min, uint64_t spin_ns, uint32_t *err)
-{
-    const bool lead = threadIdx.x == 0;
-    const int64_t nch = (lim + CH - 1) / CH;
-    StagedChunk K0 = stage_issue(T0, A, n, B, m, x0, y0, min((int64_t)CH, lim), lead);
-    StagedChunk K1{};
-    if (nch > 1)
-        K1 = stage_issue(T1, A, n, B, m, x0 + CH, y0 + CH, min((int64_t)CH, lim - CH), lead);
-    for (int64_t c = 0; c < nch; c++) {
-        const Stage T = (c & 1) ? T1 : T0;
-        const StagedChunk K = (c & 1) ? K1 : K0;
-        if (!stage_wait(T, spin_ns, err))
-            return -2;
-        const int64_t r = stage_compare(T, K, s_min);
-        if (r >= 0) {
-            // the other stage may still be receiving chunk c + 1
-            if (c + 1 < nch && !stage_wait((c & 1) ? T0 : T1, spin_ns, err))
-                return -2;
-            if (c + 1 < nch && lead)
-                *((c & 1) ? T0 : T1).phase ^= 1u;
-            __syncthreads();
-            return c * CH + r;
-        }
-        // this stage is free again: chunk c + 2 goes into it
-        if (c + 2 < nch) {
-            const StagedChunk Kn = stage_issue(T, A, n, B, m, x0 + (c + 2) * CH, y0 + (c + 2) * CH,
-                                               min((int64_t)CH, lim - (c + 2) * CH), lead);
-            if (c & 1)
-                K1 = Kn;
-            else
-                K0 = Kn;
-        }
-    }
-    return lim;
 }
 
 // ------------------------------------------------------- mod 2^61 - 1

@@ -149,8 +149,8 @@ struct LvArgs {
     // chunks of a long slide its CTA scans alone before publishing the rest
     int32_t local_chunks;
     // stages of shared memory per CTA into which bulk copies bring a long
-    // slide's chunks (0: loads into registers instead; 2: the owner streams
-    // its first chunks with the next one's copies in flight)
+    // slide's chunks (0: loads into registers instead; 2: a helper's next
+    // chunk is on its way while one is compared)
     int32_t stage;
     int32_t *wide; // the wide-band kernel's tiles: gridDim.x * lv_wide_tile_words(smax)
 };

@@ -29,12 +29,14 @@
 //  * Slides: one thread compares the two aligned 4-byte words at each start
 //    row (at least five bytes; several diagonals' loads in flight together;
 //    in the lean form 16 more bytes in one round trip when they all match);
-//    slides still open go to one warp each (ballot / first set bit over
-//    2 KiB steps), then, past t2_cap bytes, to the whole CTA, which opens a
-//    job in its job slot: 16 KiB chunks (of each string), chunk 0 scanned by
-//    the owner, the others claimed in order by atomicAdd by every CTA that is
-//    waiting on a neighbour or has no tile, each staged in shared memory by
-//    bulk copies; the first mismatch is the least over the chunks.
+//    a lean round's only open slide (the alignment path's, nearly always)
+//    goes to the whole CTA at once, several to one warp each (ballot / first
+//    set bit), then, past t2_cap bytes, to the CTA.  The CTA streams slides
+//    that run to tens of KB itself, longer ones go to a job in its job slot:
+//    chunks of 4 or 16 KiB (of each string) claimed in order by atomicAdd by
+//    every CTA that is waiting on a neighbour or has no tile, swept in
+//    registers or staged in shared memory by bulk copies; the first mismatch
+//    is the least over the chunks.
 //  * Every wait is bounded by %globaltimer and reports ST_TIMEOUT (with the
 //    place it gave up) instead of hanging.
 #include "ed_device.cuh"
@@ -231,12 +233,6 @@ __device__ __forceinline__ int64_t finish_slide(const Pair &Q, int64_t c, int64_
 }
 
 // ------------------------------------------------------------------ jobs
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p)
-{
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long *p)
 {
     unsigned long long v;
@@ -250,14 +246,6 @@ __device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned l
 // Orders the relaxed loads before it ahead of every access after it (the
 // acquire half of a flag handshake whose writer used a release).
 __device__ __forceinline__ void fence_acquire() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
-__device__ __forceinline__ void st_release_u64(unsigned long long *p, unsigned long long v)
-{
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ void set_error(const LvArgs &P, uint32_t code)
-{
-    atomicCAS(&P.ctl->error, 0u, code);
-}
 
 // A wait gave up: the first one records where (for the host's error text).
 __device__ __noinline__ void wait_failed(const LvArgs &P, unsigned long long site, unsigned long long t,
@@ -324,7 +312,6 @@ struct Smem {
     __device__ __forceinline__ unsigned long long *smin() const { return at<unsigned long long>(0); }
     __device__ __forceinline__ long long *bcl() const { return at<long long>(16); } // 4 broadcast 64-bit words
     __device__ __forceinline__ int *jring() const { return at<int>(48); } // the CTA's next job slot (0 .. JOB_RING-1)
-    __device__ __forceinline__ int *n1() const { return at<int>(64); }
     __device__ __forceinline__ int *run() const { return at<int>(72); } // mean length of its long slides (long_slide)
     __device__ __forceinline__ int *bc() const { return at<int>(80); }  // 8 broadcast words
     __device__ __forceinline__ int *jids() const { return at<int>(112); } // the job ids its slots have reached
@@ -1549,7 +1536,6 @@ __device__ __forceinline__ bool run_pair(const LvArgs &P, const Smem S, const Pa
         S.F1()[i] = NEG;
     }
     if (tid == 0) {
-        *S.n1() = 0;
         // (nothing known yet: the first slide of a string of 8 MB and more is
         // opened to other CTAs at once)
         *S.run() = (int)(min(n, m) >> 8);
