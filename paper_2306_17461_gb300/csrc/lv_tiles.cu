@@ -153,10 +153,18 @@ __device__ __noinline__ int64_t hash_lcp(const uint64_t *pow2, const HashView VA
 // The same search by a whole warp (identical arguments on every lane, the
 // answer on every lane): the doubling lengths tested at once, then the
 // bracket cut into 32 a step.  A probe waits on a round trip to the tables, so
-// that the chain of dependent probes bounds the query: about 5 here where one
+// that the chain of dependent probes bounds the query: about 5 where one
 // thread takes 2 log2(l) (28 at l = 10^4; a query took 18 us of a round's 21).
+// The search stops at a bracket [good, *bad) of BRACKET bytes: the hashes of
+// good bytes agree and those of *bad differ (*bad = good + 1 or more, or both
+// are lim), and the direct compare that confirms the answer finds the mismatch
+// in there as fast as it would confirm one place: n = 10^7, k = 1000 (three pairs):
+// 23.6 -> 16.4 ms.
+// (256 threads testing 256 to 1024 lengths a step: two trips less, and slower
+// by 5 to 33%, a table entry being a miss of HBM and of the page table.)
+constexpr int BRACKET_LOG2 = 12;
 __device__ __noinline__ int64_t hash_lcp_warp(const uint64_t *pow2, const HashView VA, const HashView VB,
-                                              int64_t x, int64_t y, int64_t lim)
+                                              int64_t x, int64_t y, int64_t lim, int64_t *bracket)
 {
     const int lane = threadIdx.x & 31;
     const uint64_t p = pow2[0];
@@ -170,6 +178,7 @@ __device__ __noinline__ int64_t hash_lcp_warp(const uint64_t *pow2, const HashVi
     const bool in = lane < 31 && L < lim;
     const unsigned int bad0 = __ballot_sync(0xffffffffu, in && !equal(L, pow2[lane]));
     int64_t good, bad = lim;
+    *bracket = lim;
     int j = __popc(__ballot_sync(0xffffffffu, in)); // lengths 2^0 .. 2^(j-1) agree
     if (bad0) {
         j = __ffs((int)bad0) - 1;
@@ -180,7 +189,7 @@ __device__ __noinline__ int64_t hash_lcp_warp(const uint64_t *pow2, const HashVi
     good = j ? 1ll << (j - 1) : 0;
     uint64_t pg = j ? pow2[j - 1] : 1ull;
     // the largest length in [good, bad) whose hashes agree, five bits a step
-    for (int k = 64 - __clzll((long long)(bad - good - 1)); k > 0;) {
+    for (int k = 64 - __clzll((long long)(bad - good - 1)); k > BRACKET_LOG2;) {
         const int step = max(k - 5, 0);
         const int64_t cand = good + ((int64_t)lane << step);
         uint64_t Pc = pg;
@@ -196,6 +205,7 @@ __device__ __noinline__ int64_t hash_lcp_warp(const uint64_t *pow2, const HashVi
         pg = __shfl_sync(0xffffffffu, Pc, f - 1);
         k = step;
     }
+    *bracket = bad;
     return good;
 }
 
@@ -210,15 +220,16 @@ struct Pair {
 
 // An open slide of diagonal d (start row c) reached row p: a mismatch at
 // p < lim_abs, or none before lim_abs (p == lim_abs).  Returns the final
-// row.  When the hash bound cut the search short and the direct compare
-// found no mismatch at the hash answer (a collision, probability about
-// l / 2^61), the slide is finished directly by this thread.
-__device__ __forceinline__ int64_t finish_slide(const Pair &Q, int64_t c, int64_t d, int64_t p,
+// row.  lo_abs, lim_abs: the hash bracket; a mismatch outside it (equal hashes
+// of different bytes: a collision, probability about l / 2^61) is counted, and
+// where the bracket cut the slide short with none found this thread finishes
+// it directly.
+__device__ __forceinline__ int64_t finish_slide(const Pair &Q, int64_t c, int64_t d, int64_t p, int64_t lo_abs,
                                                 int64_t lim_abs, bool own, Counters &C)
 {
     const int64_t full_abs = c + min(Q.n - c, Q.m - c - d);
     if (Q.hash && lim_abs < full_abs) {
-        if (own && p != lim_abs - 1)
+        if (own && (p < lo_abs || p == lim_abs))
             C.coll++;
         if (p == lim_abs) {
             bool open;
@@ -1007,18 +1018,19 @@ __device__ __forceinline__ unsigned long long *halo_ptr(const LvArgs &P, int cta
 }
 
 // The bound of an open slide of diagonal d from row c: the string end, or
-// the hash answer + 1 (the slide confirms it directly).  A whole warp calls it.
+// the end of the hash bracket that holds its mismatch (lo: its start; the slide
+// finds it directly).  A whole warp calls it.
 __device__ __forceinline__ int64_t open_limit(const LvArgs &P, const Pair &Q, int64_t c, int64_t d, Counters &C,
-                                              bool own)
+                                              bool own, int64_t &lo)
 {
     const int64_t full = min(Q.n - c, Q.m - c - d);
     int64_t lim = full;
+    lo = c;
     if (Q.hash && full > 0) {
-        const int64_t h = hash_lcp_warp(P.pow2, HashView{Q.TA, Q.A, P.hash_b}, HashView{Q.TB, Q.B, P.hash_b}, c,
-                                        c + d, full);
+        lo += hash_lcp_warp(P.pow2, HashView{Q.TA, Q.A, P.hash_b}, HashView{Q.TB, Q.B, P.hash_b}, c, c + d, full,
+                            &lim);
         if ((threadIdx.x & 31) == 0)
             C.hashq += own;
-        lim = min(h + 1, full);
     }
     return c + lim;
 }
@@ -1041,7 +1053,8 @@ __device__ __forceinline__ void warp_slides(const LvArgs &P, const Pair &Q, int3
     for (int j = w0; j < nl; j += ws) {
         const int64_t d = Ld[j], c = Lc[j];
         const bool own = d >= a && d < b;
-        const int64_t lim = open_limit(P, Q, c, d, C, own);
+        int64_t lo;
+        const int64_t lim = open_limit(P, Q, c, d, C, own, lo);
         if (lane == 0)
             C.opens += own;
         bool open;
@@ -1049,7 +1062,7 @@ __device__ __forceinline__ void warp_slides(const LvArgs &P, const Pair &Q, int3
         if (!open && l >= PREFETCH_MIN) // a long slide: the next round starts past it
             prefetch_next(Q.A, Q.n, Q.B, Q.m, c + l, c + l + d);
         if (lane == 0 && !open) {
-            fr[d - off] = (int32_t)finish_slide(Q, c, d, c + l, lim, own, C);
+            fr[d - off] = (int32_t)finish_slide(Q, c, d, c + l, lo, lim, own, C);
             Ld[j] = INT32_MIN; // finished
         }
         if (lane == 0 && open && left)
@@ -1080,7 +1093,7 @@ __device__ __forceinline__ void warp_slides(const LvArgs &P, const Pair &Q, int3
 // final rows are visible to every thread when it returns.
 __device__ __forceinline__ void cta_slides(const LvArgs &P, const Smem S, const Pair &Q, int32_t *fr, int64_t off,
                                            const int32_t *Ld, const int32_t *Lc, int nl, int64_t a, int64_t b,
-                                           Counters &C)
+                                           Counters &C, bool count = false)
 {
     const int tid = threadIdx.x;
     bool any = false;
@@ -1092,19 +1105,22 @@ __device__ __forceinline__ void cta_slides(const LvArgs &P, const Smem S, const 
         const int64_t c = Lc[j];
         const bool own = d >= a && d < b;
         if (tid < 32) {
-            const int64_t l = open_limit(P, Q, c, d, C, false);
-            if (tid == 0)
+            int64_t lo;
+            const int64_t l = open_limit(P, Q, c, d, C, count && own, lo);
+            if (tid == 0) {
+                S.bcl()[2] = lo;
                 S.bcl()[3] = l;
+            }
         }
         __syncthreads();
-        const int64_t lim = S.bcl()[3];
+        const int64_t lo = S.bcl()[2], lim = S.bcl()[3];
         __syncthreads();
         const int64_t rr = long_slide(P, S, Q, c, c + d, lim - c);
         C.longs++;
         if (tid < 32)
             prefetch_next(Q.A, Q.n, Q.B, Q.m, c + rr, c + rr + d);
         if (tid == 0)
-            fr[d - off] = (int32_t)finish_slide(Q, c, d, c + rr, lim, own, C);
+            fr[d - off] = (int32_t)finish_slide(Q, c, d, c + rr, lo, lim, own, C);
     }
     if (any) // (every thread saw the same entries)
         __syncthreads();
@@ -1317,13 +1333,13 @@ __device__ __forceinline__ void lean_slides(const LvArgs &P, const Smem S, const
         C.longs += rr >= P.t2_cap;
         if (threadIdx.x < 32) {
             if (threadIdx.x == 0) {
-                cur[d - off] = (int32_t)finish_slide(Q, c, d, c + rr, c + lim, own, C);
+                cur[d - off] = (int32_t)finish_slide(Q, c, d, c + rr, c, c + lim, own, C);
                 C.opens += own;
             }
             prefetch_next(Q.A, Q.n, Q.B, Q.m, c + rr, c + rr + d);
         }
     } else if (nlo == 1) {
-        cta_slides(P, S, Q, cur, off, Ld, Lc, nlo, a, b, C);
+        cta_slides(P, S, Q, cur, off, Ld, Lc, nlo, a, b, C, true);
     } else {
         const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
         warp_slides(P, Q, cur, off, Ld, Lc, nlo, a, b, warp, nw, C, S.left() + pr);

@@ -233,3 +233,23 @@ def test_short_pairs_on_few_ctas(ctxs, orc, n, m):
         want = orc.lv(A, B)
         for name in ctxs:
             assert ctxs[name].distance(A, B) == want, name
+
+
+@pytest.mark.parametrize("cfg", [{"lcp_mode": 2}, {"lcp_mode": 3}, {"lcp_mode": 3, "hash_block": 7}])
+def test_hash_slides_of_every_length(orc, cfg):
+    """Slides around the hash search's first lengths (eight an octave) and
+    the widths of its brackets, some to the strings' ends."""
+    from paper_2306_17461_gb300 import binding as ed
+
+    rng = np.random.default_rng(77)
+    gaps = [22, 23, 24, 31, 32, 63, 64, 95, 127, 128, 129, 1023, 1024, 1025, 1152, 8191, 8192, 8193, 9216, 16_384,
+            18_431, 40_000, 131_073, 300_000]
+    rng.shuffle(gaps)
+    pos = np.cumsum(gaps)
+    sym = W.Symbols(4)
+    A = sym.draw(rng, int(pos[-1]) + 5000)
+    B = W.plant(rng, A, pos, sym)
+    with ed.Context(device=0, **cfg) as c:
+        for X, Y in ((A, B), (A[: -4990], B), (A, A), (A[:1], A[:1]), (A, B[:-1])):
+            assert c.distance(X, Y) == orc.lv(X, Y)
+        assert c.stats()["hash_queries"] > 0
