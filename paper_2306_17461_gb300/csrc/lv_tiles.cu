@@ -155,7 +155,7 @@ __device__ __noinline__ int64_t hash_lcp(const uint64_t *pow2, const HashView VA
 // bracket cut into 32 a step.  A probe waits on a round trip to the tables, so
 // that the chain of dependent probes bounds the query: about 5 where one
 // thread takes 2 log2(l) (28 at l = 10^4; a query took 18 us of a round's 21).
-// The search stops at a bracket [good, *bad) of BRACKET bytes: the hashes of
+// The search stops at a bracket [good, *bad) of 4 KiB at most: the hashes of
 // good bytes agree and those of *bad differ (*bad = good + 1 or more, or both
 // are lim), and the direct compare that confirms the answer finds the mismatch
 // in there as fast as it would confirm one place: n = 10^7, k = 1000 (three pairs):
