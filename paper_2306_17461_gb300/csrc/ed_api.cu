@@ -1288,11 +1288,11 @@ static TileJob parked_job(ed_ctx *ctx, const BatchPair &b)
 // chain, but the longest job bounds the launch: a job that would take more
 // than half of what the whole set takes on all CTAs (one and a half times
 // that while the groups leave CTAs free) gets a group twice as large, down to
-// WIDE_TILE_MIN diagonals a CTA (64 served pairs: 79 ms with 512, 75 with 1024,
-// 93 with 2048; the batch of 4096 pairs does not care).  A single job takes the whole grid, and while
+// WIDE_TILE_MIN diagonals a CTA (1024: 64 served pairs 79 -> 75 ms, but another
+// set of 29 20.6 -> 22.7 ms; 2048: 93 ms).  A single job takes the whole grid, and while
 // the groups fill at most half of it they are doubled.
 constexpr double WIDE_ROUND_US = 2.0, WIDE_DIAG_US = 0.75e-3;
-constexpr int64_t WIDE_TILE_MIN = 1024;
+constexpr int64_t WIDE_TILE_MIN = 512;
 static void spread_jobs(ed_ctx *ctx, std::vector<TileJob> &jobs)
 {
     if (jobs.size() == 1)

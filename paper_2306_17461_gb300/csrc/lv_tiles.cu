@@ -323,6 +323,7 @@ struct Smem {
     __device__ __forceinline__ unsigned long long *smin() const { return at<unsigned long long>(0); }
     __device__ __forceinline__ long long *bcl() const { return at<long long>(16); } // 4 broadcast 64-bit words
     __device__ __forceinline__ int *jring() const { return at<int>(48); } // the CTA's next job slot (0 .. JOB_RING-1)
+    __device__ __forceinline__ int *from() const { return at<int>(64); } // where the CTA looks for open jobs first
     __device__ __forceinline__ int *run() const { return at<int>(72); } // mean length of its long slides (long_slide)
     __device__ __forceinline__ int *bc() const { return at<int>(80); }  // 8 broadcast words
     __device__ __forceinline__ int *jids() const { return at<int>(112); } // the job ids its slots have reached
@@ -611,6 +612,8 @@ __device__ int claim_loop2(const LvArgs &P, const Smem S, JobSlot *sl, int s, in
             // 1. the claim in flight: valid, worth a scan?
             const int nv = wn && claim_valid(P, wn) ? 1 : 0;
             const int ng = nv ? claim_go(P, S, sl, s, wn, bestn, made + pvalid == 0 ? pre : nullptr) : 0;
+            if (nv && !ng)
+                *S.from() = s + 1;
             const unsigned long long wc = wn;
             // 2. its copies, in flight while the pending chunk is compared
             if (ng && S.jd()->chunk > SMALL_CHUNK) {
@@ -674,9 +677,12 @@ __device__ int claim_loop2(const LvArgs &P, const Smem S, JobSlot *sl, int s, in
 }
 
 // Thread 0: an open job slot of another CTA, or -1.  The active bitmask
-// over the slots (its first eight words loaded together) is read from a
-// CTA-dependent bit on, so that helpers spread over jobs.
-__device__ __forceinline__ int pick_slot(const LvArgs &P)
+// over the slots (its first eight words loaded together) is read from bit
+// `from` on: a CTA-dependent one at first, so that helpers spread over jobs,
+// and past a job whose chunks were all claimed when the CTA came to it, so that
+// jobs of several CTAs (the path's slide in its neighbours' halos) are served
+// together and not one after the other's last answer.
+__device__ __forceinline__ int pick_slot(const LvArgs &P, int from)
 {
     int s = -1;
     const int nslot = (int)gridDim.x * JOB_RING;
@@ -686,8 +692,7 @@ __device__ __forceinline__ int pick_slot(const LvArgs &P)
 #pragma unroll
     for (int k = 0; k < 8; k++)
         b[k] = k < nw ? act[k] : 0ull;
-    const int rot = blockIdx.x & 63;
-    const int w0 = (int)(((int)blockIdx.x * JOB_RING / 64) % nw);
+    const int rot = from & 63, w0 = (from >> 6) % nw;
     for (int k = 0; k < nw && s < 0; k++) {
         const int wd = (w0 + k) % nw;
         unsigned long long v = 0ull;
@@ -864,6 +869,7 @@ __device__ __noinline__ int64_t run_job(const LvArgs &P, const Smem S, const Pai
 constexpr int64_t ALONE_BYTES = 64 * 1024;
 constexpr int RUN_BYTES = 32 * 1024;
 constexpr int SMALL_RUN = 256 * 1024;
+constexpr int SMALL_SPAN = 128; // small chunks of one slide
 __device__ __noinline__ int64_t long_slide(const LvArgs &P, const Smem S, const Pair Q, int64_t x0,
                                            int64_t y0, int64_t lim0)
 {
@@ -877,8 +883,10 @@ __device__ __noinline__ int64_t long_slide(const LvArgs &P, const Smem S, const 
     while (r < 0 && off < lim0) {
         // slides that run to a few hundred KB go in small chunks, one load a
         // thread: more CTAs share them, and a chunk takes half as long
-        const bool small = mean <= SMALL_RUN;
-        const int64_t len = min(lim0 - off, (int64_t)JOB_MAX_CHUNKS * chunk_bytes(small));
+        // (their first 512 KiB, a chunk for nearly every CTA: a slide that
+        // goes on past that is not one of them)
+        const bool small = mean <= SMALL_RUN && off == loc;
+        const int64_t len = min(lim0 - off, (int64_t)(small ? SMALL_SPAN : JOB_MAX_CHUNKS) * chunk_bytes(small));
         const int64_t q = run_job(P, S, Q, x0 + off, y0 + off, len, small);
         if (q < len)
             r = off + q;
@@ -1315,18 +1323,22 @@ __device__ __forceinline__ BlockOut run_block(const LvArgs &P, const Smem S, con
 }
 
 // The open slides of a lean round (out of line: most rounds have none): a
-// lone one goes to the whole CTA at once (it matched 21 bytes and more: the
-// alignment path's, nearly always, of n / k bytes; a warp's step first, up to
-// t2_cap bytes, cost 2 thousand cycles when it fell short and gained nothing
-// when it did not: n = 10^6, k = 500, slides of 2 KB, 1.88 -> 1.53 ms), several
-// to one warp each, then to the whole CTA those still open.  Every thread calls
-// it (after a barrier); the final rows are visible to every thread when it
-// returns.
+// lone one (the alignment path's, nearly always, of n / k bytes) goes to the
+// whole CTA at once while the running mean of the long slides is SHORT_RUN and
+// more -- a warp's step first cost 2 thousand cycles when it fell short and
+// gained nothing when it did not: n = 10^6, k = 500, slides of 2 KB, 1.88 ->
+// 1.53 ms -- and to a warp below it, which ends slides of a few dozen bytes with
+// less ceremony (n = 38 thousand, k = 882: 4.6 ms by the CTA, 4.1 by a warp; at
+// 10^3 bytes the CTA is ahead, 6.8 against 7.3).  Several go to one warp each,
+// then to the whole CTA those still open.  Every thread calls it (after a
+// barrier); the final rows are visible to every thread when it returns.
+constexpr int SHORT_RUN = 512;
 __device__ __forceinline__ void lean_slides(const LvArgs &P, const Smem S, const Pair Q, int32_t *cur, int64_t off,
                                          int32_t *Ld, const int32_t *Lc, int nlo, int64_t a, int64_t b, int pr,
                                          Counters &C)
 {
-    if (nlo == 1 && !Q.hash) {
+    const bool direct = nlo == 1 && *S.run() >= SHORT_RUN;
+    if (direct && !Q.hash) {
         const int64_t d = Ld[0], c = Lc[0], lim = min(Q.n - c, Q.m - c - d);
         const bool own = d >= a && d < b;
         const int64_t rr = long_slide(P, S, Q, c, c + d, lim);
@@ -1338,14 +1350,17 @@ __device__ __forceinline__ void lean_slides(const LvArgs &P, const Smem S, const
             }
             prefetch_next(Q.A, Q.n, Q.B, Q.m, c + rr, c + rr + d);
         }
-    } else if (nlo == 1) {
+    } else if (direct) {
         cta_slides(P, S, Q, cur, off, Ld, Lc, nlo, a, b, C, true);
     } else {
         const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        const int32_t d0 = Ld[0]; // (thread 0's: its warp takes the entry and marks it)
         warp_slides(P, Q, cur, off, Ld, Lc, nlo, a, b, warp, nw, C, S.left() + pr);
         __syncthreads();
         if (S.left()[pr])
             cta_slides(P, S, Q, cur, off, Ld, Lc, nlo, a, b, C);
+        else if (threadIdx.x == 0 && nlo == 1) // (long_slide counts the others)
+            *S.run() += (cur[d0 - off] - Lc[0] - *S.run()) >> 2;
         if (threadIdx.x == 0)
             S.left()[pr] = 0;
     }
@@ -1598,7 +1613,7 @@ __device__ __forceinline__ bool run_pair(const LvArgs &P, const Smem S, const Pa
                         const uint32_t er = *(volatile uint32_t *)&P.ctl->error;
                         const uint32_t eq = *(volatile uint32_t *)&gc->epoch_req;
                         const uint32_t ec = *(volatile uint32_t *)&gc->ebar_count;
-                        const int js = pick_slot(P);
+                        const int js = pick_slot(P, *S.from());
                         // a job of the group is served even once the epoch
                         // change is asked for, until every tile is at the
                         // barrier (no job of the group opens after that)
@@ -1826,7 +1841,7 @@ __device__ __forceinline__ bool run_pair(const LvArgs &P, const Smem S, const Pa
                         v[u] = (jj < h && wp) ? ld_relaxed_u64(wp + jj) : ~0ull;
                     }
                     // an open job of another CTA, looked for in the same round trip
-                    int q = tid == 0 ? pick_slot(P) : -1;
+                    int q = tid == 0 ? pick_slot(P, *S.from()) : -1;
 #pragma unroll
                     for (int u = 0; u < HMAX / 16; u++)
                         ok = ok && (uint32_t)(v[u] >> 32) >= tag;
@@ -1924,6 +1939,7 @@ __global__ void __launch_bounds__(CTA_THREADS, 1) lv_tiles_kernel(LvArgs P)
         S.jd()->slot = -1;
         S.jd()->pq = -1;
         *S.jring() = 0;
+        *S.from() = (int)blockIdx.x * JOB_RING;
         for (int i = 0; i < JOB_RING; i++)
             S.jids()[i] = (int)P.jid0;
         for (int i = 0; i < 4; i++)

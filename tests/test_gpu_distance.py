@@ -253,3 +253,21 @@ def test_hash_slides_of_every_length(orc, cfg):
         for X, Y in ((A, B), (A[: -4990], B), (A, A), (A[:1], A[:1]), (A, B[:-1])):
             assert c.distance(X, Y) == orc.lv(X, Y)
         assert c.stats()["hash_queries"] > 0
+
+
+@pytest.mark.parametrize("cfg", [{"block_rounds": 64, "tile_width": 16, "help_div": -1}, {"block_rounds": 64, "local_chunks": 2}])
+def test_jobs_of_several_ctas_at_once(orc, cfg):
+    """The path's slide runs in its neighbours' halos as well: their jobs are
+    open together.  Slides short (a warp's), of several small-chunk spans, and
+    of a length the running mean does not expect."""
+    from paper_2306_17461_gb300 import binding as ed
+
+    rng = np.random.default_rng(78)
+    pos = np.cumsum([1_300_000, 30, 50, 30, 40, 50, 60, 40, 30, 600_000, 520_000, 530_000, 20, 1_100_000])
+    sym = W.Symbols(4)
+    A = sym.draw(rng, int(pos[-1]) + 700_000)
+    B = W.plant(rng, A, pos, sym)
+    want = orc.lv(A, B)
+    with ed.Context(device=0, **cfg) as c:
+        for _ in range(3):
+            assert c.distance(A, B) == want
