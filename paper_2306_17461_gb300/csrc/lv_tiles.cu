@@ -159,7 +159,7 @@ __device__ __noinline__ int64_t hash_lcp(const uint64_t *pow2, const HashView VA
 // good bytes agree and those of *bad differ (*bad = good + 1 or more, or both
 // are lim), and the direct compare that confirms the answer finds the mismatch
 // in there as fast as it would confirm one place: n = 10^7, k = 1000 (three pairs):
-// 23.6 -> 16.4 ms.
+// 23.6 -> 17.0 ms.
 // (256 threads testing 256 to 1024 lengths a step: two trips less, and slower
 // by 5 to 33%, a table entry being a miss of HBM and of the page table.)
 constexpr int BRACKET_LOG2 = 12;
@@ -587,7 +587,7 @@ __device__ int claim_loop(const LvArgs &P, const Smem S, JobSlot *sl, int s, uns
 // The same claims, answers and stopping rules as claim_loop, but a CTA with
 // nothing pending takes one small chunk only, and answers it at once: such jobs
 // are short, and a chunk queued behind another was their last answer (slides of
-// 10^5 bytes: 6.7 -> 6.0 us a round).
+// 10^5 bytes: 6.7 -> 6.2 us a round).
 __device__ int claim_loop2(const LvArgs &P, const Smem S, JobSlot *sl, int s, int budget, const Wake *wake)
 {
     const int tid = threadIdx.x;
@@ -1327,7 +1327,7 @@ __device__ __forceinline__ BlockOut run_block(const LvArgs &P, const Smem S, con
 // whole CTA at once while the running mean of the long slides is SHORT_RUN and
 // more -- a warp's step first cost 2 thousand cycles when it fell short and
 // gained nothing when it did not: n = 10^6, k = 500, slides of 2 KB, 1.88 ->
-// 1.53 ms -- and to a warp below it, which ends slides of a few dozen bytes with
+// 1.55 ms -- and to a warp below it, which ends slides of a few dozen bytes with
 // less ceremony (n = 38 thousand, k = 882: 4.6 ms by the CTA, 4.1 by a warp; at
 // 10^3 bytes the CTA is ahead, 6.8 against 7.3).  Several go to one warp each,
 // then to the whole CTA those still open.  Every thread calls it (after a
