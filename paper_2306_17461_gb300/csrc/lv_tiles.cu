@@ -365,7 +365,7 @@ struct Smem {
 // its last job, and nothing is cleared.  The owner publishes with plain
 // relaxed stores (a release waited 2 thousand cycles for them): a claimer
 // whose claim ran ahead of the descriptor sees an older job's id in it and
-// looks again.  A claim that lands on a job published after the claimer
+// looks again, and in the end leaves the chunk to the owner.  A claim that lands on a job published after the claimer
 // looked is a claim of that job.
 //   ans[c]  = (jid << 32) | job offset of the chunk's first mismatch (NOMIS: none)
 //   result  = (jid << 32) | ~best  (so that red.max keeps the least offset)
@@ -403,15 +403,19 @@ __device__ __forceinline__ void answer_claim(JobSlot *sl, uint32_t jid, int64_t 
         red_max_u64(&sl->ans[c], tg | (r >= 0 ? (uint32_t)r : NOMIS));
 }
 
-// Thread 0, after a claim w of slot s: whether its chunk is worth scanning
-// (inside lim and below the best mismatch reported so far).  The job's
-// descriptor is read into the CTA's cache once per job, after a fence that
-// orders it behind the claim: x, y, lim and the pair (whose strings the
-// launch's pair table holds), each word tagged with its job; words of
-// another job mean the slot has moved on (the claim's job is over: nothing
-// to scan).  best: the result word read along with the claim (~0: read it
-// here).  A descriptor outside its strings is never scanned (self-check
-// record 7).
+// Thread 0, after a claim w of slot s: 1 when its chunk is worth scanning, 0
+// when it is not (past lim, or past the best mismatch reported so far: answered
+// without a look), -1 when the claim must be left without an answer.  The job's
+// descriptor is read into the CTA's cache once per job: x, y, lim and the pair
+// (whose strings the launch's pair table holds), each word tagged with its job.
+// Words of a later job mean that the claim's job is over: nobody waits for the
+// answer.  Words of an older one mean that the descriptor is still on its way:
+// they are looked at again, CLAIM_LOOKS times at most, and then the chunk is
+// left to the job's owner, which compares a claimed chunk that does not answer
+// itself.  (An answer here would call bytes equal that nobody has compared.)
+// best: the result word read along with the claim (~0: read it here).  A
+// descriptor outside its strings is never scanned (self-check record 7).
+constexpr int CLAIM_LOOKS = 256;
 __device__ __forceinline__ int claim_go(const LvArgs &P, const Smem S, JobSlot *sl, int s, unsigned long long w,
                                         unsigned long long best = ~0ull, const unsigned long long *pre = nullptr)
 {
@@ -420,8 +424,8 @@ __device__ __forceinline__ int claim_go(const LvArgs &P, const Smem S, JobSlot *
     JobDesc *J = S.jd();
     if (J->jid != jid || J->slot != s) {
         // the words read along with the claim serve when they all carry its
-        // job (each word holds its tag with its value); else read them again
-        // behind a fence
+        // job (each word holds its tag with its value); else they are read
+        // again
         unsigned long long xt = 0, yt = 0, lt = 0, pt = 0;
         bool tags = false;
         if (pre) {
@@ -441,13 +445,8 @@ __device__ __forceinline__ int claim_go(const LvArgs &P, const Smem S, JobSlot *
             const uint32_t t0 = (uint32_t)(xt >> 32), t1 = (uint32_t)(yt >> 32), t2 = (uint32_t)(lt >> 32),
                            t3 = (uint32_t)(pt >> 32), t4 = (uint32_t)(best >> 32);
             tags = t0 == jid && t1 == jid && t2 == jid && t3 == jid && t4 >= jid;
-            // a later job's word: the claim's job is over; an older one's: the
-            // descriptor is still on its way (looked at again, a bounded number
-            // of times: the owner scans a chunk that nobody answers)
-            if (!tags && (max(max(t0, t1), max(t2, t3)) > jid || look == 256)) {
-                J->jid = 0;
-                return 0;
-            }
+            if (!tags && (max(max(t0, t1), max(t2, t3)) > jid || look == CLAIM_LOOKS))
+                return -1; // (the cached job, if any, stays as it is)
         }
         // the pair's strings: the launch's pair table, read once per pair
         const uint32_t pi = (uint32_t)pt & PAIR_MASK;
@@ -477,7 +476,7 @@ __device__ __forceinline__ int claim_go(const LvArgs &P, const Smem S, JobSlot *
                 P.ctl->diag[5] = (unsigned long long)J->n;
                 P.ctl->diag[6] = (unsigned long long)J->m;
             }
-            return 0;
+            return -1;
         }
     } else if (best == ~0ull) {
         best = ld_relaxed_u64(&sl->result);
@@ -537,10 +536,10 @@ __device__ __forceinline__ bool wake_ready(const Wake *w)
 // `budget` claims: thread 0 makes the next claim before the current chunk
 // is scanned, so that its round trip overlaps the scan.  w0: a claim made
 // already (0: make the first one here).  Stops once a claimed chunk lies
-// past the end or past the best mismatch, or its job is over (that claim is
-// answered at once), or, with a Wake, once the CTA's neighbours are ready
-// (checked along with each claim).  Returns the number of claims made and
-// answered.
+// past the end or past the best mismatch (that claim is answered at once), or
+// must be left unanswered (claim_go), or, with a Wake, once the CTA's neighbours
+// are ready (checked along with each claim).  Returns the number of claims made
+// and answered.
 __device__ int claim_loop(const LvArgs &P, const Smem S, JobSlot *sl, int s, unsigned long long w0, int budget,
                           const Wake *wake = nullptr, unsigned long long best0 = ~0ull)
 {
@@ -553,15 +552,14 @@ __device__ int claim_loop(const LvArgs &P, const Smem S, JobSlot *sl, int s, uns
     for (;;) {
         if (tid == 0) {
             const bool ready = wake && wake_ready(wake);
-            const int valid = claim_valid(P, w) ? 1 : 0;
-            const int go = valid ? claim_go(P, S, sl, s, w, best) : 0;
-            S.bc()[0] = valid;
+            const int go = claim_valid(P, w) ? claim_go(P, S, sl, s, w, best) : -1;
+            S.bc()[0] = go >= 0;
             S.bc()[3] = go;
             S.bcl()[0] = (long long)w;
             // the next claim and a look at the result, both in flight during
             // the scan below (this claim is still unanswered: the job cannot
             // change meanwhile)
-            const bool next = go && !ready && made + 1 < budget;
+            const bool next = go > 0 && !ready && made + 1 < budget;
             w = next ? atomicAdd(&sl->claim, 1ull) : 0ull;
             best = next ? ld_relaxed_u64(&sl->result) : ~0ull;
             S.bc()[4] = next;
@@ -609,10 +607,11 @@ __device__ int claim_loop2(const LvArgs &P, const Smem S, JobSlot *sl, int s, in
     for (;;) {
         const int sn = ps ^ 1;   // the stage for the claim resolved this turn
         if (tid == 0) {
-            // 1. the claim in flight: valid, worth a scan?
-            const int nv = wn && claim_valid(P, wn) ? 1 : 0;
-            const int ng = nv ? claim_go(P, S, sl, s, wn, bestn, made + pvalid == 0 ? pre : nullptr) : 0;
-            if (nv && !ng)
+            // 1. the claim in flight: to be answered, worth a scan?
+            const bool live = wn && claim_valid(P, wn);
+            const int go = live ? claim_go(P, S, sl, s, wn, bestn, made + pvalid == 0 ? pre : nullptr) : -1;
+            const int nv = go >= 0, ng = go > 0;
+            if (live && !ng)
                 *S.from() = s + 1;
             const unsigned long long wc = wn;
             // 2. its copies, in flight while the pending chunk is compared
