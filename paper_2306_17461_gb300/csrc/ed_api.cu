@@ -265,7 +265,7 @@ struct ed_ctx {
         border, bnext, bfront, keep, wtiles;
     char *h_ctl = nullptr; // pinned image of a tile launch's control block
     size_t h_ctl_cap = 0;
-    bool slots_used = false; // every id in the slots is at most next_jid
+    bool slots_used = false; // the slots are cleared or used: every id in them is at most next_jid
     uint32_t next_jid = 0;
     // pinned staging of short host strings (HostPacker): two halves, each busy
     // until its event
@@ -546,10 +546,14 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
     P.cls_p0[ncls] = pi;
     P.ncls = ncls;
     const int grid = cta;
-    const DevBuf slots0 = ctx->slots;
+    // (new slots are not cleared yet: whatever fails from here on, the next
+    // launch clears them)
+    const size_t slot_bytes = sizeof(JobSlot) * grid * JOB_RING;
+    if (!wide && ctx->slots.bytes < slot_bytes)
+        ctx->slots_used = false;
     if ((r = ensure(ctx, ctx->gf, sizeof(int32_t) * (size_t)std::max<int64_t>(gf_total, 1))) != ED_OK ||
         (wide && (r = ensure(ctx, ctx->wtiles, sizeof(int32_t) * grid * lv_wide_tile_words((int)smax))) != ED_OK) ||
-        (!wide && (r = ensure(ctx, ctx->slots, sizeof(JobSlot) * grid * JOB_RING)) != ED_OK) ||
+        (!wide && (r = ensure(ctx, ctx->slots, slot_bytes)) != ED_OK) ||
         (r = ensure(ctx, ctx->halo, sizeof(unsigned long long) * (size_t)grid * 4 * HMAX)) != ED_OK)
         return r;
     // the launch's control words in one block, written by one copy and read
@@ -624,8 +628,7 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
         // job ids go on from the last launch's, so that the slots' old words
         // (10 MB of them) need no clearing; they are cleared when new, when
         // another call wrote them, after a failed launch and before ids run out
-        if (!ctx->slots_used || ctx->slots.p != slots0.p || ctx->slots.bytes != slots0.bytes ||
-            ctx->next_jid >= 1u << 30) {
+        if (!ctx->slots_used || ctx->next_jid >= 1u << 30) {
             CK(cudaMemsetAsync(ctx->slots.p, 0, ctx->slots.bytes, s));
             ctx->next_jid = 0;
         }

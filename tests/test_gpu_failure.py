@@ -107,3 +107,32 @@ def test_serving_refuses_admission_on_memory_then_admits(orc):
         assert ed.ed_serve_counters(c.h)["admitted"] == 2
     finally:
         c.close()
+
+
+def test_slots_new_in_a_failed_call_are_cleared(orc):
+    """A call that fails after the job slots have grown (no room for the edge
+    words that come next) leaves slots that were never cleared; the next call
+    must not take what lies in them for answers.  The memory they land in holds
+    words that read as "no mismatch" of the first jobs."""
+    import torch
+
+    from paper_2306_17461_gb300 import binding as ed
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    keep, gf = 4 * (2 * 600_000 + 5), 8 * (2 * 2048 * sms + 5)  # of a pair of 600 thousand characters
+    slots, edges = 2 * sms * 33_024, 2048 * sms
+    short, mid, far, last = (W.make_pair(140 + i, n, k, sigma=4)
+                             for i, (n, k) in enumerate([(1500, 4), (600_000, 2), (4_000_000, 2), (300_000, 2)]))
+    with ed.Context(device=0, mem_budget_bytes=keep + gf + slots + edges * 5 // 8) as c:
+        assert c.distance_dev(dev(short.A), dev(short.B)) == orc.lv(short.A, short.B)
+        bufs = [(dev(p.A), dev(p.B)) for p in (mid, far, last)]
+        words = (torch.arange(8 << 20, device="cuda") % 8 + 1) << 32 | 0xFFFFFFFF
+        torch.cuda.synchronize()
+        del words
+        torch.cuda.empty_cache()
+        for a, b in bufs[:2]:  # no room for the edge words, then for the frontier (which gives its room back)
+            with pytest.raises(ed.EdError) as ei:
+                c.distance_dev(a, b)
+            assert ei.value.code == ed.ED_ENOMEM
+        assert c.distance_dev(*bufs[2]) == orc.lv(last.A, last.B)
+        assert c.stats()["long_slides"] >= 1
