@@ -132,6 +132,7 @@ struct Request {
     // resident frontier (keep, radius keep_r) and the round / radius to
     // resume from (t0 = 0: from the start)
     int tile_G = 0;
+    bool narrow = false; // on the tile kernel: the budget had no room for the wide-band kernel's tiles
     double cost = 0.0;
     char *keep = nullptr;
     size_t bytesK = 0;
@@ -159,6 +160,7 @@ struct TileJob {
     // L1/shared memory to the L1, which holds the rows' string bytes.
     int64_t smax_want = 0;
     bool wide = false; // on the wide-band kernel (every job of a launch alike)
+    int g0 = 1; // wide-band jobs: the smallest group that holds the estimated band
 };
 
 // What a tile launch left for one pair: its distance (st 0), or ST_WIDE,
@@ -345,6 +347,17 @@ void release(ed_ctx *ctx, DevBuf &b)
     b.bytes = 0;
 }
 
+// Whether the budget has room for these buffers at (at least) these sizes, as
+// ensure would make them one after another.
+bool room_for(const ed_ctx *ctx, std::initializer_list<std::pair<const DevBuf *, size_t>> want)
+{
+    size_t more = 0;
+    for (const auto &w : want)
+        if (w.second > w.first->bytes)
+            more += std::max(w.second, (size_t)4096) - w.first->bytes;
+    return ctx->held + more <= ctx->budget;
+}
+
 int status_from_kernel(uint32_t st)
 {
     if (st == 0)
@@ -431,27 +444,18 @@ int run_hash_tables(ed_ctx *ctx, const uint8_t *dA, int64_t n, const uint8_t *dB
     return ED_OK;
 }
 
-// One tile launch over the jobs, CTA groups by class (one class per group
-// size wanted).  Every class that fits gets one group, largest first; the
-// remaining CTAs go, one group at a time, to the class whose estimated run
-// time per group is highest.  out[i] receives each pair's outcome; the
-// counters of pairs that finished or were suspended are summed into
+// One tile launch over the jobs on at most maxg CTAs, in groups by class (one
+// class per group size wanted).  Every class that fits gets one group, largest
+// first; the remaining CTAs go, one group at a time, to the class whose
+// estimated run time per group is highest.  out[i] receives each pair's outcome;
+// the counters of pairs that finished or were suspended are summed into
 // ctx->last.  budget_ns > 0 time-slices the pairs that have a keep buffer.
-static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStream_t s, uint64_t budget_ns,
-                          std::vector<TileOut> &out)
+static int tile_launch(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStream_t s, uint64_t budget_ns, int maxg,
+                       std::vector<TileOut> &out)
 {
     int r;
     const int np = (int)jobs.size();
     const bool wide = jobs[0].wide;
-    int maxg = wide ? ctx->wgrid : ctx->grid;
-    if (wide) { // no more CTAs than the memory budget has room for their tiles
-        int64_t nm = 1;
-        for (const TileJob &j : jobs)
-            nm = std::max(nm, std::max(j.n, j.m));
-        const size_t per = sizeof(int32_t) * lv_wide_tile_words((int)std::min<int64_t>(SMAX_LIMIT, 2 * nm + 2));
-        while (maxg > 1 && per * maxg > ctx->wtiles.bytes && ctx->held - ctx->wtiles.bytes + per * maxg > ctx->budget)
-            maxg = (maxg + 1) / 2;
-    }
     const int h = ctx->eff.block_rounds;
     const int s0 = ctx->eff.tile_width;
     // classes, ascending group size; pairs by class, then cost, largest first
@@ -546,16 +550,6 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
     P.cls_p0[ncls] = pi;
     P.ncls = ncls;
     const int grid = cta;
-    // (new slots are not cleared yet: whatever fails from here on, the next
-    // launch clears them)
-    const size_t slot_bytes = sizeof(JobSlot) * grid * JOB_RING;
-    if (!wide && ctx->slots.bytes < slot_bytes)
-        ctx->slots_used = false;
-    if ((r = ensure(ctx, ctx->gf, sizeof(int32_t) * (size_t)std::max<int64_t>(gf_total, 1))) != ED_OK ||
-        (wide && (r = ensure(ctx, ctx->wtiles, sizeof(int32_t) * grid * lv_wide_tile_words((int)smax))) != ED_OK) ||
-        (!wide && (r = ensure(ctx, ctx->slots, slot_bytes)) != ED_OK) ||
-        (r = ensure(ctx, ctx->halo, sizeof(unsigned long long) * (size_t)grid * 4 * HMAX)) != ED_OK)
-        return r;
     // the launch's control words in one block, written by one copy and read
     // back (from the launch's words on) by another: groups, pairs, launch,
     // results
@@ -563,7 +557,19 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
     const size_t o_ctl = (o_pairs + sizeof(PairDesc) * np + 63) & ~(size_t)63;
     const size_t o_res = o_ctl + sizeof(LaunchCtl);
     const size_t block = o_res + sizeof(unsigned long long) * R_COUNT * np;
-    if ((r = ensure(ctx, ctx->ctl, block)) != ED_OK)
+    const size_t gf_bytes = sizeof(int32_t) * (size_t)std::max<int64_t>(gf_total, 1);
+    const size_t tile_bytes = wide ? sizeof(int32_t) * grid * lv_wide_tile_words((int)smax) : 0;
+    const size_t halo_bytes = sizeof(unsigned long long) * (size_t)grid * 4 * HMAX;
+    if (wide && !room_for(ctx, {{&ctx->gf, gf_bytes}, {&ctx->wtiles, tile_bytes}, {&ctx->halo, halo_bytes}, {&ctx->ctl, block}}))
+        return ED_ENOMEM; // (nothing given back: the caller asks for less)
+    // (new slots are not cleared yet: whatever fails from here on, the next
+    // launch clears them)
+    const size_t slot_bytes = sizeof(JobSlot) * grid * JOB_RING;
+    if (!wide && ctx->slots.bytes < slot_bytes)
+        ctx->slots_used = false;
+    if ((r = ensure(ctx, ctx->gf, gf_bytes)) != ED_OK || (wide && (r = ensure(ctx, ctx->wtiles, tile_bytes)) != ED_OK) ||
+        (!wide && (r = ensure(ctx, ctx->slots, slot_bytes)) != ED_OK) ||
+        (r = ensure(ctx, ctx->halo, halo_bytes)) != ED_OK || (r = ensure(ctx, ctx->ctl, block)) != ED_OK)
         return r;
     if (ctx->h_ctl_cap < block) {
         if (ctx->h_ctl)
@@ -694,26 +700,73 @@ static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStr
     return ED_OK;
 }
 
-// Runs pairs on the tile kernel until each has its distance: a pair whose
-// band outgrew its group runs again on a group twice as large; a pair
-// that needs more than the whole grid, or more rounds than the cap, fails
-// the call with ED_ELIMIT.
-int run_tiles(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStream_t s, std::vector<uint64_t> &k)
+// tile_launch on the kernel's whole grid.  The wide-band kernel's tiles lie in
+// the context's memory: when its budget has no room for them, on half as many
+// CTAs, and so on.  *maxg: the CTAs there was room for.
+static int run_tiles_once(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStream_t s, uint64_t budget_ns,
+                          std::vector<TileOut> &out, int *maxg)
+{
+    for (*maxg = jobs[0].wide ? ctx->wgrid : ctx->grid;; *maxg = (*maxg + 1) / 2) {
+        const int r = tile_launch(ctx, jobs, s, budget_ns, *maxg, out);
+        if (r != ED_ENOMEM || !jobs[0].wide || *maxg == 1)
+            return r;
+    }
+}
+
+// Wide-band jobs whose tiles the memory budget does not hold go to the tile
+// kernel, whose tiles lie in shared memory: what the wide-band kernel's launches
+// hold is given back.
+static void give_up_wide(ed_ctx *ctx)
+{
+    if (!ctx->wtiles.p)
+        return;
+    release(ctx, ctx->wtiles);
+    release(ctx, ctx->gf);
+}
+
+// Runs pairs on the tile kernel or (wide jobs) the wide-band kernel until each
+// has its distance: a pair whose band outgrew its group runs again on a group
+// twice as large; a pair that needs more than the whole grid, or more rounds
+// than the cap, fails the call with ED_ELIMIT.  Wide jobs that need more than
+// the memory budget has tiles for run on the tile kernel instead, from round 0
+// (their init is taken out of jobs).
+int run_tiles(ed_ctx *ctx, std::vector<TileJob> &jobs, cudaStream_t s, std::vector<uint64_t> &k)
 {
     k.assign(jobs.size(), 0);
-    std::vector<TileJob> cur = jobs;
-    std::vector<size_t> idx(jobs.size());
+    std::vector<TileJob> cur = jobs, narrow;
+    std::vector<size_t> idx(jobs.size()), narrow_idx;
     for (size_t i = 0; i < idx.size(); i++)
         idx[i] = i;
-    while (!cur.empty()) {
+    auto to_narrow = [&](const TileJob &j, size_t i) {
+        TileJob q = j;
+        q.wide = false;
+        q.G = std::min(ctx->grid, q.g0);
+        q.init = jobs[i].init = nullptr;
+        narrow.push_back(q);
+        narrow_idx.push_back(i);
+    };
+    while (!cur.empty() || !narrow.empty()) {
+        if (cur.empty()) { // the wide jobs are done
+            give_up_wide(ctx);
+            cur.swap(narrow);
+            idx.swap(narrow_idx);
+        }
         std::vector<TileOut> o;
-        int r = run_tiles_once(ctx, cur, s, 0, o);
+        const bool wide = cur[0].wide;
+        int maxg = 0;
+        int r = run_tiles_once(ctx, cur, s, 0, o, &maxg);
+        if (r == ED_ENOMEM && wide) {
+            for (size_t i = 0; i < cur.size(); i++)
+                to_narrow(cur[i], idx[i]);
+            cur.clear();
+            idx.clear();
+            continue;
+        }
         if (r != ED_OK)
             return r;
         std::vector<TileJob> next;
         std::vector<size_t> nidx;
         for (size_t i = 0; i < cur.size(); i++) {
-            const int maxg = cur[i].wide ? ctx->wgrid : ctx->grid;
             if (o[i].st == 0) {
                 k[idx[i]] = o[i].k;
             } else if (o[i].st == ST_WIDE &&
@@ -730,6 +783,8 @@ int run_tiles(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStream_t s, std
                 j.R0 = resume ? o[i].rr : 0;
                 next.push_back(j);
                 nidx.push_back(idx[i]);
+            } else if (o[i].st == ST_WIDE && wide && maxg < ctx->wgrid) {
+                to_narrow(cur[i], idx[i]);
             } else {
                 char buf[160];
                 std::snprintf(buf, sizeof(buf), "pair %zu: %s", idx[i],
@@ -767,7 +822,8 @@ int run_pair(ed_ctx *ctx, const uint8_t *dA, int64_t n, const uint8_t *dB, int64
         j.TB = (const uint64_t *)ctx->hashB.p;
     }
     std::vector<uint64_t> k;
-    if ((r = run_tiles(ctx, {j}, s, k)) != ED_OK)
+    std::vector<TileJob> jobs = {j};
+    if ((r = run_tiles(ctx, jobs, s, k)) != ED_OK)
         return r;
     if (hash_mode(ctx)) {
         float bms = 0.f;
@@ -1279,7 +1335,7 @@ static TileJob parked_job(ed_ctx *ctx, const BatchPair &b)
     const int64_t band = std::min<int64_t>(2 * (kest + kest / 4) + 1, b.n + b.m + 1);
     while (j.G < ctx->wgrid && (int64_t)j.G * SMAX_LIMIT < band)
         j.G *= 2;
-    j.G = std::min(j.G, ctx->wgrid);
+    j.G = j.g0 = std::min(j.G, ctx->wgrid);
     return j;
 }
 
@@ -1388,17 +1444,21 @@ static int batch_core(ed_ctx *ctx, size_t np, const uint8_t *const *A, const siz
         for (size_t p : parked) {
             const BatchPair &b = hp[p];
             jobs.push_back(parked_job(ctx, b));
-            ext += count_extensions(b.n, b.m, b.t); // its rounds so far
-            slide += b.slide;
-            mism += b.mism;
         }
         spread_jobs(ctx, jobs);
         ctx->last = ed_stats{};
         std::vector<uint64_t> kk;
         if ((r = run_tiles(ctx, jobs, s, kk)) != ED_OK)
             return r;
-        for (size_t i = 0; i < parked.size(); i++)
+        for (size_t i = 0; i < parked.size(); i++) {
+            const BatchPair &b = hp[parked[i]];
             k_out[parked[i]] = kk[i];
+            if (jobs[i].init) { // the batch kernel's rounds, which it went on from
+                ext += count_extensions(b.n, b.m, b.t);
+                slide += b.slide;
+                mism += b.mism;
+            }
+        }
         ext += ctx->last.extensions;
         slide += ctx->last.slide_chars;
         mism += ctx->last.compared_bytes / 2 - ctx->last.slide_chars;
@@ -1646,20 +1706,23 @@ static void engine_loop(ed_ctx *ctx)
         // (2) the tile kernel, time-sliced
         std::vector<size_t> tidx;
         std::vector<TileJob> jobs;
+        // (once one needs the tile kernel, all run there: the two kernels'
+        // buffers are not held together)
+        const bool narrow = std::any_of(ctx->live.begin(), ctx->live.end(), [](const Request *q) { return q->narrow; });
         for (size_t i = 0; i < L; i++) {
             Request *q = ctx->live[i];
             if (!q->tile_G || done[i])
                 continue;
             TileJob j{(const uint8_t *)q->dA, (const uint8_t *)q->dB, q->n, q->m, nullptr, nullptr, nullptr, 0,
                       q->tile_G, q->cost};
-            j.init = (const int32_t *)q->front;
+            j.init = narrow ? nullptr : (const int32_t *)q->front;
             j.init_t = q->t + 1;
             j.init_zero = BATCH_W / 2 + 1;
             j.keep = (int32_t *)q->keep;
             j.keep_r = q->keep ? q->keep_r : 0;
             j.t0 = q->keep ? q->t0 : 0;
             j.R0 = q->R0;
-            j.wide = true;
+            j.wide = !narrow;
             tidx.push_back(i);
             jobs.push_back(j);
         }
@@ -1667,13 +1730,19 @@ static void engine_loop(ed_ctx *ctx)
             // each pair's group at least what its band needs (tile_G), all of
             // them spread over the grid (a single pair takes all of it: its
             // resident frontier holds any group's band)
-            if (std::all_of(jobs.begin(), jobs.end(), [](const TileJob &j) { return j.keep != nullptr; }))
+            if (!narrow &&
+                std::all_of(jobs.begin(), jobs.end(), [](const TileJob &j) { return j.keep != nullptr; }))
                 spread_jobs(ctx, jobs);
+            if (narrow)
+                give_up_wide(ctx);
             std::vector<TileOut> o;
-            const int rt = run_tiles_once(ctx, jobs, ctx->sstream, SERVE_TILE_NS, o);
+            int maxg = 0;
+            const int rt = run_tiles_once(ctx, jobs, ctx->sstream, SERVE_TILE_NS, o, &maxg);
             for (size_t j = 0; j < tidx.size(); j++) {
                 Request *q = ctx->live[tidx[j]];
-                if (rt != ED_OK) {
+                if (rt == ED_ENOMEM && !narrow) {
+                    q->narrow = true;
+                } else if (rt != ED_OK) {
                     result[tidx[j]] = rt;
                     done[tidx[j]] = 1;
                 } else if (o[j].st == 0) {
@@ -1683,13 +1752,20 @@ static void engine_loop(ed_ctx *ctx)
                     q->t0 = o[j].rt;
                     q->R0 = o[j].rr;
                     ctx->n_slices++;
-                } else if (o[j].st == ST_WIDE && q->keep && o[j].rt > 0 && jobs[j].G < ctx->wgrid) {
+                } else if (o[j].st == ST_WIDE && q->keep && o[j].rt > 0 && jobs[j].G < maxg) {
                     // a larger group from the saved round
-                    q->tile_G = std::min(ctx->wgrid, 2 * jobs[j].G);
+                    q->tile_G = std::min(maxg, 2 * jobs[j].G);
                     q->t0 = o[j].rt;
                     q->R0 = o[j].rr;
-                } else if (o[j].st == ST_WIDE && q->tile_G < ctx->wgrid) {
-                    to_tiles(ctx, q, std::min(ctx->wgrid, 2 * q->tile_G)); // again, from round 0
+                } else if (o[j].st == ST_WIDE && q->tile_G < maxg) {
+                    // again, from the batch kernel's round (on the tile kernel: from round 0)
+                    to_tiles(ctx, q, std::min(maxg, 2 * q->tile_G));
+                } else if (o[j].st == ST_WIDE && !narrow && maxg < ctx->wgrid) {
+                    q->narrow = true;
+                    if (q->keep && o[j].rt > 0) {
+                        q->t0 = o[j].rt;
+                        q->R0 = o[j].rr;
+                    }
                 } else {
                     result[tidx[j]] = ED_ELIMIT;
                     done[tidx[j]] = 1;

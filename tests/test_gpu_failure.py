@@ -136,3 +136,40 @@ def test_slots_new_in_a_failed_call_are_cleared(orc):
             assert ei.value.code == ed.ED_ENOMEM
         assert c.distance_dev(*bufs[2]) == orc.lv(last.A, last.B)
         assert c.stats()["long_slides"] >= 1
+
+
+@pytest.mark.timeout(300)
+@pytest.mark.parametrize("call", ["batch", "served"])
+def test_wide_band_under_every_budget(orc, call):
+    """A pair whose band (40001 diagonals) is wider than two of its four CTAs
+    hold: whatever the memory budget, the call gives the distance or says that
+    memory is short.  What the pair takes with its tiles in shared memory (job
+    slots, re-tiling buffers, the batch kernel's frontier, edges and control
+    words) is enough."""
+    from paper_2306_17461_gb300 import binding as ed
+
+    n = 20_000
+    rng = W.rng_for(303, 0)
+    A, B = W.Symbols(4).draw(rng, n), W.Symbols(4).draw(rng, n) + 4
+    want = orc.lv(A, B)
+    assert 2 * want + 1 > 2 * 16_384
+    dA, dB = dev(A), dev(B)
+    enough = 4 * 2 * 33_024 + 16 * (n + 5) + 4 * 4_099 + 4 * 2_048 + 8 * 4_096
+    base = 0 if call == "batch" else 64 << 20  # the arena's smallest size
+    short = 0
+    for budget in list(range(64 << 10, enough, 48 << 10)) + [enough + i * (48 << 10) for i in range(12)]:
+        with ed.Context(device=0, grid_ctas=4, mem_budget_bytes=base + budget) as c:
+            try:
+                if call == "batch":
+                    k = int(ed.ed_distance_batch_dev(c.h, [dA], [dB])[0])
+                else:
+                    ticket = ed.ed_submit(c.h, A, B)
+                    st = ed.ED_EAGAIN
+                    while st == ed.ED_EAGAIN:
+                        st, k = ed.ed_poll(c.h, ticket)
+                        time.sleep(0.001)
+                assert k == want, budget
+            except ed.EdError as e:
+                assert e.code == ed.ED_ENOMEM and budget < enough, (budget, str(e))
+                short += 1
+    assert short > 0
