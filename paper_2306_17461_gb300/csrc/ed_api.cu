@@ -518,6 +518,13 @@ static int tile_launch(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStream
         kcap = std::min<int64_t>(kcap, ctx->cfg.max_rounds);
     kcap = std::min<int64_t>(kcap, (int64_t)1 << 28);
     kcap = std::max<int64_t>(kcap, h);
+    // Under the cap a pair ends with the last block of h rounds that ends by
+    // round kcap, counted from round 0.  Wide-band jobs start their blocks at
+    // the batch kernel's round: their kernel runs as far as that round takes it,
+    // and a distance beyond the cap's last round is refused below.
+    const int64_t klast = (kcap + 1) / h * h - 1, kask = kcap;
+    if (wide)
+        kcap = klast + h - 1;
     // tile capacity: what the widest band of any class needs, at most SMAX_LIMIT
     // (a group also runs pairs of the classes below its own)
     int64_t smax = std::max(h, s0), nm_below = 0, want_below = 0;
@@ -678,6 +685,9 @@ static int tile_launch(ed_ctx *ctx, const std::vector<TileJob> &jobs, cudaStream
             // rounds from .. rt - 1 done in this launch
             ctx->last.extensions += count_extensions(jobs[i].n, jobs[i].m, o.rt - 1) - before;
         } else if (o.st != 0) {
+            continue;
+        } else if (wide && kask < std::max(jobs[i].n, jobs[i].m) && (int64_t)R[R_K] > klast) {
+            o.st = ST_LIMIT;
             continue;
         } else {
             o.k = R[R_K];

@@ -4,6 +4,8 @@ several strips, groups of one and of several CTAs, block lengths that do not
 divide the segments, strings at every alignment, ends reached early (unequal
 lengths, one symbol), and slides that outrun their warp.  Integer results: the
 tolerance is zero."""
+import time
+
 import numpy as np
 import pytest
 
@@ -64,3 +66,30 @@ def test_wide_bands_match_oracle(pairs, cfg):
         assert np.array_equal(got, want), cfg
         again = ed.ed_distance_batch_dev(c.h, dB, dA)  # the strings exchanged
         assert np.array_equal(again, want), cfg
+
+
+@pytest.mark.parametrize("call", ["batch", "served"])
+@pytest.mark.parametrize("h", [32, 5, 64])
+def test_round_cap(orc, h, call):
+    """max_rounds counts whole blocks of h rounds from round 0, wherever the
+    batch kernel left the pair: a cap that ends the block holding round k
+    gives the distance, one less is refused."""
+    from paper_2306_17461_gb300 import binding as ed
+
+    A, B = W.random_pair(np.random.default_rng(304), 24_000, 3100, 256)
+    k = orc.lv(A, B)
+    assert k > 2048
+    cap = (k // h + 1) * h - 1
+    for rounds in (cap, cap - 1, 2080):
+        with ed.Context(device=0, block_rounds=h, max_rounds=rounds) as c:
+            try:
+                if call == "batch":
+                    got = int(ed.ed_distance_batch_dev(c.h, [dev(A)], [dev(B)])[0])
+                else:
+                    t, st = ed.ed_submit(c.h, A, B), ed.ED_EAGAIN
+                    while st == ed.ED_EAGAIN:
+                        st, got = ed.ed_poll(c.h, t)
+                        time.sleep(0.001)
+            except ed.EdError as e:
+                got = e.code
+        assert got == (k if rounds == cap else ed.ED_ELIMIT), rounds
