@@ -440,7 +440,7 @@ int run_hash_tables(ed_ctx *ctx, const uint8_t *dA, int64_t n, const uint8_t *dB
         return r;
     CK(launch_prefix_hash(dA, n, ctx->hash_base, (uint64_t *)ctx->hashA.p, b, ctx->scan.p, s));
     CK(launch_prefix_hash(dB, m, ctx->hash_base, (uint64_t *)ctx->hashB.p, b, ctx->scan.p, s));
-    ctx->last.kernel_launches += 2;
+    ctx->last.kernel_launches += prefix_hash_launches(n) + prefix_hash_launches(m);
     return ED_OK;
 }
 

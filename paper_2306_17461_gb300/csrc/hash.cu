@@ -48,6 +48,8 @@ size_t prefix_hash_state_bytes(int64_t len)
     return 2 * sizeof(uint64_t) * (size_t)tiles; // each tile's hash, and the prefix before it
 }
 
+int prefix_hash_launches(int64_t len) { return len > TILE_CHARS ? 3 : 1; }
+
 // A multiplier b as mul61 takes it: b and b * 2^32 mod q, each hi * 2^31 + lo.
 struct Mul61 {
     uint32_t c0l, c0h, c1l, c1h;

@@ -218,5 +218,6 @@ cudaError_t launch_lcp_queries(const uint8_t *A, int64_t n, const uint8_t *B, in
 cudaError_t launch_prefix_hash(const uint8_t *X, int64_t len, uint64_t base, uint64_t *T, int64_t stride,
                                void *scan_state, cudaStream_t s);
 size_t prefix_hash_state_bytes(int64_t len);
+int prefix_hash_launches(int64_t len); // kernels of one launch_prefix_hash
 
 } // namespace edg

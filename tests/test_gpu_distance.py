@@ -271,3 +271,15 @@ def test_jobs_of_several_ctas_at_once(orc, cfg):
     with ed.Context(device=0, **cfg) as c:
         for _ in range(3):
             assert c.distance(A, B) == want
+
+
+@pytest.mark.parametrize("n,m", [(16_384, 16_384), (16_384, 16_385), (16_385, 16_384), (40_000, 40_000)])
+def test_launches_counted_with_hash_tables(orc, n, m):
+    """A prefix table is one launch up to 16384 characters and three beyond."""
+    from paper_2306_17461_gb300 import binding as ed
+
+    A = np.random.default_rng(79).integers(0, 4, max(n, m), dtype=np.uint8)
+    for cfg in ({"lcp_mode": 2}, {"lcp_mode": 3}):
+        with ed.Context(device=0, **cfg) as c:
+            assert c.distance(A[:n], A[:m]) == orc.lv(A[:n], A[:m])
+            assert c.stats()["kernel_launches"] == 1 + sum(3 if x > 16_384 else 1 for x in (n, m))
