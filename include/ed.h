@@ -97,7 +97,9 @@ typedef struct {
     uint64_t extensions;     /* diagonal-extensions: (t, d) cells evaluated */
     uint64_t slide_chars;    /* sum over extensions of the LCP length */
     uint64_t compared_bytes; /* 2 * (slide_chars + mismatching compares) */
-    uint64_t long_slides;    /* slides handed to the job slots (helped) */
+    uint64_t long_slides;    /* slides of warp_cap bytes and more, answered by
+                                a whole CTA and, when longer still, by the
+                                CTAs that help it through the job slots */
     uint64_t open_slides;    /* slides the start-row words did not finish
                                 (continued by a warp), tile kernel only */
     uint64_t wide_rounds;    /* rounds run in temporal blocks */

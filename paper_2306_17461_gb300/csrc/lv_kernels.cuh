@@ -94,7 +94,7 @@ enum {
     R_K = 0,
     R_SLIDE = 1,      // sum of LCP lengths
     R_MISMATCH = 2,   // slides that ended on a mismatching pair
-    R_LONG = 3,       // slides given to the job slots
+    R_LONG = 3,       // slides of t2_cap bytes and more
     R_WIDE = 4,       // temporal blocks run
     R_HASHQ = 5,
     R_HASHCOLL = 6,

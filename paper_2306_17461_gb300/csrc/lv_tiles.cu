@@ -1097,10 +1097,12 @@ __device__ __forceinline__ void warp_slides(const LvArgs &P, const Pair &Q, int3
 
 // The listed slides a warp left open: the whole CTA each (and beyond 128
 // KiB the job slots).  Every thread must call it, after a barrier; the
-// final rows are visible to every thread when it returns.
+// final rows are visible to every thread when it returns.  first: no warp has
+// tried them (their hash queries are counted here, and only those of t2_cap
+// bytes and more as long).
 __device__ __forceinline__ void cta_slides(const LvArgs &P, const Smem S, const Pair &Q, int32_t *fr, int64_t off,
                                            const int32_t *Ld, const int32_t *Lc, int nl, int64_t a, int64_t b,
-                                           Counters &C, bool count = false)
+                                           Counters &C, bool first = false)
 {
     const int tid = threadIdx.x;
     bool any = false;
@@ -1113,7 +1115,7 @@ __device__ __forceinline__ void cta_slides(const LvArgs &P, const Smem S, const 
         const bool own = d >= a && d < b;
         if (tid < 32) {
             int64_t lo;
-            const int64_t l = open_limit(P, Q, c, d, C, count && own, lo);
+            const int64_t l = open_limit(P, Q, c, d, C, first && own, lo);
             if (tid == 0) {
                 S.bcl()[2] = lo;
                 S.bcl()[3] = l;
@@ -1123,7 +1125,7 @@ __device__ __forceinline__ void cta_slides(const LvArgs &P, const Smem S, const 
         const int64_t lo = S.bcl()[2], lim = S.bcl()[3];
         __syncthreads();
         const int64_t rr = long_slide(P, S, Q, c, c + d, lim - c);
-        C.longs++;
+        C.longs += !first || rr >= P.t2_cap;
         if (tid < 32)
             prefetch_next(Q.A, Q.n, Q.B, Q.m, c + rr, c + rr + d);
         if (tid == 0)

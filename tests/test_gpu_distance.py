@@ -283,3 +283,20 @@ def test_launches_counted_with_hash_tables(orc, n, m):
         with ed.Context(device=0, **cfg) as c:
             assert c.distance(A[:n], A[:m]) == orc.lv(A[:n], A[:m])
             assert c.stats()["kernel_launches"] == 1 + sum(3 if x > 16_384 else 1 for x in (n, m))
+
+
+@pytest.mark.parametrize("lcp_mode", [1, 2, 3])
+def test_long_slides_are_those_past_warp_cap(orc, lcp_mode):
+    """long_slides counts slides of warp_cap bytes (4096) and more, however
+    they were answered: none of 2 KB, every one of 20 KB."""
+    from paper_2306_17461_gb300 import binding as ed
+
+    rng = np.random.default_rng(80)
+    sym = W.Symbols(4)
+    for gap, edits in ((2000, 100), (20_000, 12)):
+        A = sym.draw(rng, gap * (edits + 1))
+        B = W.plant(rng, A, gap * np.arange(1, edits + 1), sym)
+        with ed.Context(device=0, lcp_mode=lcp_mode, help_div=-1) as c:
+            assert c.distance(A, B) == orc.lv(A, B)
+            st = c.stats()
+            assert st["long_slides"] == 0 if gap < 4096 else st["long_slides"] >= edits, (gap, st["long_slides"])
