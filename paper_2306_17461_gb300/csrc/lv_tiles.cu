@@ -355,6 +355,11 @@ struct Smem {
     }
 };
 
+// (the header's parts end where the next one starts)
+static_assert(JOB_RING <= (128 - 112) / (int)sizeof(int), "the job ids fill bytes 112..127 of the shared memory");
+static_assert(sizeof(JobDesc) <= 256 - 192, "the job cache fills bytes 192..255");
+static_assert(256 + 4 * sizeof(unsigned long long) <= HEADER, "the phase times lie below the frontier buffers");
+
 // Job slot protocol.  claim = (job id << 32) | count: every atomicAdd of 1
 // claims chunk `count` (CHUNK_BYTES of each string) of the job the word
 // names.  The job's descriptor words and every word a claimer writes back
