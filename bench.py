@@ -213,7 +213,7 @@ REGIME = {
     "small": "round latency (n = 1e6 fits in L2; 1e2 rounds)",
     "mid_k10": "HBM streaming: ten slides of about 1e7 bytes each",
     "mid_k1000": "round chain: every round waits on the path's slide of about 1e5 bytes",
-    "mid_k100000": "scattered start-row loads of 2e5 diagonals a round (L1 throughput)",
+    "mid_k100000": "the alignment path's CTA: its slide and 1300 diagonals a round; the others wait for it",
     "large": "round chain: 1e4 sequential rounds, a slide of about 2e6 bytes after each burst",
 }
 

@@ -64,7 +64,8 @@ typedef struct {
     int lcp_mode;             /* ed_lcp_mode */
     uint64_t hash_seed;       /* selects the hash base; 0 = fixed default */
     uint64_t spin_limit_ns;   /* bound of every device-side wait; 0 = 2e9 */
-    int grid_ctas;            /* CTAs of the tile kernel; 0 = one per SM */
+    int grid_ctas;            /* CTAs of the tile and wide-band kernels;
+                                 0 = one per SM */
     int tile_width;           /* diagonals per CTA in the first epoch (the
                                  tiles grow with the band, by an eighth at
                                  a time); 0 = 64 */
@@ -75,10 +76,14 @@ typedef struct {
     int hash_block;           /* block size b of ED_LCP_BHASH (1..4096);
                                  0 = 32 */
     int warp_cap;             /* bytes one warp compares before a slide
-                                 goes to the whole CTA (>= 512); 0 = 4096 */
-    int local_chunks;         /* 16 KiB chunks a CTA compares alone before
-                                 its long slide is opened to other CTAs;
-                                 0 = none (open at once) */
+                                 goes to the whole CTA (>= 512); 0 = 4096.
+                                 (A round's only open slide goes to the CTA
+                                 at once while slides run to 512 bytes.) */
+    int local_chunks;         /* 16 KiB chunks a CTA compares alone, at
+                                 least, before its long slide is opened to
+                                 other CTAs; 0 = none asked for (while
+                                 slides run to 32 KiB at most, it is 64 KiB
+                                 all the same) */
     int help_div;             /* while the band is narrow, 1/help_div of a
                                  group's CTAs hold no tile and serve long
                                  slides; 0 = 8, -1 = none */
@@ -101,7 +106,8 @@ typedef struct {
                                 a whole CTA and, when longer still, by the
                                 CTAs that help it through the job slots */
     uint64_t open_slides;    /* slides the start-row words did not finish
-                                (continued by a warp), tile kernel only */
+                                (continued by a warp or the CTA); not the
+                                batch kernel's */
     uint64_t wide_rounds;    /* rounds run in temporal blocks */
     uint64_t hash_queries;   /* LCP queries answered by the hash search */
     uint64_t hash_collisions;/* hash answers refuted by the direct check */
@@ -164,7 +170,7 @@ int ed_last_stats(ed_ctx *ctx, ed_stats *out);
  * DEVICE pointers of lengths n[p], m[p] (the pointer arrays themselves are
  * host arrays); k_out is a host array of npairs entries.  One persistent
  * launch claims pairs from a cost-ordered work queue; pairs whose band
- * outgrows one CTA continue on the single-pair kernel.  Synchronous. */
+ * outgrows one CTA continue on the wide-band kernel.  Synchronous. */
 int ed_distance_batch_dev(ed_ctx *ctx, size_t npairs,
                           const uint8_t *const *A, const size_t *n,
                           const uint8_t *const *B, const size_t *m,
@@ -200,7 +206,7 @@ int ed_submit_dev(ed_ctx *ctx, const uint8_t *A, size_t n, const uint8_t *B,
                   size_t m, uint64_t *ticket, void *stream);
 
 /* Serving counters: admitted, completed, in flight, engine steps, and
- * slices (times a pair on the tile kernel was left at a sync point with its
+ * slices (times a pair on the wide-band kernel was left at a sync point with its
  * band frontier saved, to be resumed at the next step).  Null pointers are
  * skipped. */
 int ed_serve_counters(ed_ctx *ctx, uint64_t *admitted, uint64_t *completed,

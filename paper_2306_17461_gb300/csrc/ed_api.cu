@@ -39,7 +39,9 @@ constexpr int START_TILE = 2048; // diagonals per CTA a single pair starts with
 // streams their slides as fast as others would help, their widest band is 171
 // diagonals a CTA, and the group's barriers, its skipping tiles and the end of
 // the pair wait for 24 CTAs instead of 152.  n = 10^3, k = 13: 95 -> 83 us a call,
-// k = 27: 105 -> 95 us, k = 80: 150 -> 133 us.  (On longer strings the same is
+// k = 27: 105 -> 95 us, k = 80: 150 -> 133 us; unrelated strings of 2 KB (k near
+// n, the widest band) take 1322 us here and 1271 on the whole grid, which a rule
+// by length cannot tell apart beforehand.  (On longer strings the same is
 // gained for k < 100, but a band of thousands of diagonals wants the whole
 // grid, and moving it there costs 100 us.  8 CTAs and fewer, 32 and more: slower.)
 constexpr int FEW_CTAS = 24;
@@ -128,9 +130,9 @@ struct Request {
     cudaEvent_t ready = nullptr;
     int64_t n = 0, m = 0;
     int32_t t = -1;
-    // on the tile kernel (band wider than one batch CTA): its group size,
+    // on the wide-band kernel (band wider than one batch CTA): its group size,
     // resident frontier (keep, radius keep_r) and the round / radius to
-    // resume from (t0 = 0: from the start)
+    // resume from (t0 = 0: from the batch kernel's round)
     int tile_G = 0;
     bool narrow = false; // on the tile kernel: the budget had no room for the wide-band kernel's tiles
     double cost = 0.0;
@@ -139,7 +141,7 @@ struct Request {
     int64_t keep_r = 0, t0 = 0, R0 = 0;
 };
 
-// One pair handed to the tile kernel.
+// One pair handed to the tile kernel or (wide) the wide-band kernel.
 struct TileJob {
     const uint8_t *A, *B;
     int64_t n, m;
@@ -810,7 +812,8 @@ int run_tiles(ed_ctx *ctx, std::vector<TileJob> &jobs, cudaStream_t s, std::vect
     return ED_OK;
 }
 
-// One pair, device strings, on stream s (the whole grid as one group).
+// One pair, device strings, on stream s (the whole grid as one group; short
+// pairs on FEW_CTAS).
 int run_pair(ed_ctx *ctx, const uint8_t *dA, int64_t n, const uint8_t *dB, int64_t m,
              cudaStream_t s, int32_t *dump, int64_t dump_tmax, uint64_t *k_out)
 {
@@ -1448,8 +1451,8 @@ static int batch_core(ed_ctx *ctx, size_t np, const uint8_t *const *A, const siz
     }
     ed_stats keep = ctx->last;
     if (!parked.empty()) {
-        // pairs whose band outgrew one CTA: CTA groups of the tile kernel,
-        // sized by each pair's estimated distance, in one launch
+        // pairs whose band outgrew one CTA: CTA groups of the wide-band
+        // kernel, sized by each pair's estimated distance, in one launch
         std::vector<TileJob> jobs;
         for (size_t p : parked) {
             const BatchPair &b = hp[p];
@@ -1600,7 +1603,7 @@ int ed_distance_batch(ed_ctx *ctx, size_t np, const uint8_t *const *A, const siz
 
 // ------------------------------------------------------------------ serving
 // Device time per engine step: the batch kernel (pairs within one CTA's
-// band), then the tile kernel (pairs whose band outgrew it).
+// band), then the wide-band kernel (pairs whose band outgrew it).
 constexpr uint64_t SERVE_BATCH_NS = 2000000;
 constexpr uint64_t SERVE_TILE_NS = 4000000;
 
@@ -1617,7 +1620,7 @@ static void release_request(ed_ctx *ctx, Request *q)
     q->ready = nullptr;
 }
 
-// Moves a request to the tile kernel on a group of G CTAs, with a resident
+// Moves a request to the wide-band kernel on a group of G CTAs, with a resident
 // frontier as wide as the whole grid's tiles (so that the pair can change
 // groups between steps; none if the arena is full: the pair then runs to
 // its end in one launch).
@@ -1632,11 +1635,11 @@ static void to_tiles(ed_ctx *ctx, Request *q, int G)
     q->R0 = 0;
 }
 
-// One engine step: the live pairs not yet on the tile kernel get up to
+// One engine step: the live pairs not yet on the wide-band kernel get up to
 // SERVE_BATCH_NS in one launch of the batch kernel (frontiers resident in
-// the arena); those whose band outgrew a CTA move to the tile kernel, where
-// every such pair gets up to SERVE_TILE_NS per step and its band frontier
-// stays resident between steps.
+// the arena); those whose band outgrew a CTA move to the wide-band kernel (to
+// the tile kernel when memory is short), where every such pair gets up to
+// SERVE_TILE_NS per step and its band frontier stays resident between steps.
 static void engine_loop(ed_ctx *ctx)
 {
     cudaSetDevice(ctx->device);
@@ -1699,8 +1702,6 @@ static void engine_loop(ed_ctx *ctx)
                     result[bidx[j]] = b.k;
                     done[bidx[j]] = 1;
                 } else if (b.state == 2) {
-                    // group from the distance estimate, doubled while the
-                    // tile pairs would fill at most half of the grid
                     // the group its estimated band needs; each step spreads
                     // the groups over the grid
                     const TileJob pj = parked_job(ctx, b);
@@ -1713,7 +1714,7 @@ static void engine_loop(ed_ctx *ctx)
             }
         }
         ctx->n_steps++;
-        // (2) the tile kernel, time-sliced
+        // (2) the wide-band kernel, time-sliced
         std::vector<size_t> tidx;
         std::vector<TileJob> jobs;
         // (once one needs the tile kernel, all run there: the two kernels'

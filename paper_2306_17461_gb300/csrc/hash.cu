@@ -259,6 +259,9 @@ __global__ void __launch_bounds__(HT, HPER_SM) prefix_hash_kernel(const uint8_t 
         // row's end, summed over lanes 0 .. 7
         if (r + 1 < HROWS) {
             uint64_t e = lane < HW ? fold61(mul61(s_warp[r & 1][lane], mend)) : 0ull;
+            // (they fit in 64 bits: lane 7's multiplier is 1 and its value below
+            // 2^61; the others are at most 2^61, as fold61 takes values below
+            // 2^62 + 2^34 to at most that)
 #pragma unroll
             for (int o = 4; o; o >>= 1)
                 e += __shfl_xor_sync(0xffffffffu, e, o);

@@ -5,7 +5,7 @@
 // frontier in shared memory: per round, the shared round function (several
 // diagonals' loads in flight per thread), then the open slides, one warp
 // each, then the whole CTA for those still open.  A pair whose band outgrows
-// W diagonals is parked (state 2) for the tile kernel.  With a time budget
+// W diagonals is parked (state 2) for the wide-band kernel.  With a time budget
 // (serving), a CTA stops a pair at a round boundary once the budget is
 // spent, saves the round's frontier in the pair's resident buffer, and the
 // next launch resumes it.

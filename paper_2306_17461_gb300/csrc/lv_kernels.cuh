@@ -50,7 +50,7 @@ struct PairDesc {
     int32_t *dump;             // frontier dump (tests) or null
     int32_t dump_tmax;
     int32_t pad;
-    // resident frontier across launches (serving) or null: L_{t-1}[d] at
+    // resident frontier across launches (serving, wider tiles) or null: L_{t-1}[d] at
     // keep[d + keep_r + 2] for |d| <= keep_r; the pair starts at round t0
     // with epoch radius R0 when t0 > 0
     int32_t *keep;
@@ -170,7 +170,7 @@ struct BatchPair {
     int64_t n, m;
     int32_t *front;    // W + 3 int32: the pair's resident frontier (round t)
     int32_t t;         // rounds completed so far (-1 = not started)
-    int32_t state;     // 0 running, 1 done, 2 needs the tile kernel, 3 self-check failed
+    int32_t state;     // 0 running, 1 done, 2 needs the wide-band kernel, 3 self-check failed
     int64_t k;
     int64_t reach;     // when parked: the furthest row of the saved frontier
     unsigned long long slide, mism;

@@ -492,8 +492,9 @@ __device__ __forceinline__ int claim_go(const LvArgs &P, const Smem S, JobSlot *
 
 // The first mismatch of A[x0..x0+len) vs B[y0..) (len <= CHUNK_BYTES), or
 // -1: by bulk copies into the CTA's stage when it has one, else (and for small
-// chunks) by register sweeps.  Whole CTA.  (A stage wait that gave up has set the launch status; the chunk then counts as
-// equal and the launch reports the timeout.)
+// chunks) by register sweeps.  Whole CTA.  (A stage wait that gave up has set
+// the launch status; the chunk then counts as equal and the launch reports the
+// timeout.)
 __device__ __forceinline__ int64_t chunk_scan(const LvArgs &P, const Smem S, const uint8_t *A, int64_t n,
                                               const uint8_t *B, int64_t m, int64_t x0, int64_t y0, int64_t len)
 {
@@ -1100,8 +1101,8 @@ __device__ __forceinline__ void warp_slides(const LvArgs &P, const Pair &Q, int3
     }
 }
 
-// The listed slides a warp left open: the whole CTA each (and beyond 128
-// KiB the job slots).  Every thread must call it, after a barrier; the
+// The listed slides a warp left open: the whole CTA each (and, as they run
+// longer, the job slots: long_slide).  Every thread must call it, after a barrier; the
 // final rows are visible to every thread when it returns.  first: no warp has
 // tried them (their hash queries are counted here, and only those of t2_cap
 // bytes and more as long).

@@ -3,11 +3,19 @@
 // frontier and the strings' bytes at it in registers (lv_window.cuh).
 //
 // The single-pair kernel of lv_tiles.cu is built for narrow bands: rounds
-// bound by their latency, long slides spread over idle CTAs.  A pair whose
-// band has outgrown its narrow tiles is left by that kernel at a block's end
-// with the band's frontier saved, and goes on here; batched and served pairs
-// whose band has outgrown one CTA of the batch kernel run here from the
-// start.  What bounds these rounds is the integer work of their diagonals.
+// bound by their latency, long slides spread over idle CTAs.  Batched and
+// served pairs whose band has outgrown one CTA of the batch kernel go on here
+// from its frontier; single pairs stay there, however wide (n = 10^8, k = 10^5
+// handed over at 386 diagonals a CTA: 303 to 308 ms against 288).
+//
+// What bounds these rounds: the warps wait for one another.  152 pairs of
+// 40 thousand characters, k = 6400, one CTA each (45 ms, 2.5 cycles a diagonal
+// and SM; over a mixed batch it is about 1.45): 42 % of a warp's time at the
+// CTA's barriers (a warp with the path's slide or a checked round holds up the
+// other 15, by the code), 20 % for its own last instruction; a scheduler of
+// four warps issues in 42 % of its cycles, the integer pipe is busy 43 %, L1
+// 17 %, and HBM not at all.  With the halo, the warps' overlap and the checked
+// rounds a diagonal takes 123 instructions.
 //
 // GB300 mapping.
 //  * A group of CTAs splits the diagonals [-R, R] into one tile per CTA; R (the epoch radius) grows by an eighth

@@ -82,7 +82,7 @@ __device__ __forceinline__ uint32_t first_byte(uint32_t x) // index of the lowes
 //
 // No clamp, no bound and no band test here: a row this far from both ends
 // cannot be clamped, and a slot outside the band has a negative row.  About
-// 35 integer operations a slot; the integer pipe bounds it.
+// 35 integer operations a slot (what bounds the rounds: lv_wide.cu).
 template <int E>
 __device__ __forceinline__ bool fast_round(Win<E> &w, int32_t x1, int32_t x2, const WinString &U, const WinString &V,
                                            int32_t delta, uint32_t &slide, uint32_t &open)

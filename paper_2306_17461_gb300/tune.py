@@ -12,7 +12,8 @@ measured once):
     block_rounds  rounds between neighbour exchanges
     tile_width    diagonals per CTA in the first epoch
     warp_cap      bytes one warp compares before the whole CTA takes a slide
-    local_chunks  16 KiB chunks a CTA compares alone before opening a slide
+                  (one of several in a round, or while slides are short)
+    local_chunks  16 KiB chunks a CTA compares alone, at least, before opening a slide
     help_div      1/help_div of the CTAs serve long slides while the band is narrow
     lcp_mode      direct comparison, or the prefix-hash search of Sec. 3.2 /
                   Alg. 2 (blocked tables), every hash answer confirmed
