@@ -10,7 +10,7 @@
 //
 // What bounds these rounds: the warps wait for one another.  152 pairs of
 // 40 thousand characters, k = 6400, one CTA each (45 ms, 2.5 cycles a diagonal
-// and SM; over a mixed batch it is about 1.45): 42 % of a warp's time at the
+// and SM; 1.8 in the rounds of a batch of 4096, on groups of CTAs): 42 % of a warp's time at the
 // CTA's barriers (a warp with the path's slide or a checked round holds up the
 // other 15, by the code), 20 % for its own last instruction; a scheduler of
 // four warps issues in 42 % of its cycles, the integer pipe is busy 43 %, L1
@@ -18,8 +18,9 @@
 // rounds a diagonal takes 123 instructions.
 //
 // GB300 mapping.
-//  * A group of CTAs splits the diagonals [-R, R] into one tile per CTA; R (the epoch radius) grows by an eighth
-//    and the tiles are then cut again through a global buffer.
+//  * A group of CTAs splits the diagonals [-R, R] into one tile per CTA; R (the
+//    epoch radius) grows by an eighth and the tiles are then cut again through
+//    a global buffer.
 //  * Temporal blocking: a CTA runs h rounds on its tile plus h halo diagonals
 //    a side, then trades h edge values with its neighbours through global
 //    memory, each in one 8-byte word with its round (no fence, no flag).
